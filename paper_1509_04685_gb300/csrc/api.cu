@@ -259,7 +259,7 @@ int cola_init(const cola_config* cfg, void* ws, size_t ws_bytes, void* stream) {
     if (cudaMemsetAsync(ws, 0, kHdrBytes, s) != cudaSuccess) return COLA_ECUDA;
     if ((rc = launch_twiddles(twiddle_ptr(ws, kTwMesh), cfg->ng, s))) return rc;
     if ((rc = launch_twiddles(twiddle_ptr(ws, kTwLagr), cfg->nq, s))) return rc;
-    return launch_tables(cfg, table_ptr(ws), s);
+    return launch_tables(cfg, table_ptr(ws), growth_ptr(ws), s);
 }
 
 int cola_ic_2lpt(const cola_config* cfg, uint64_t seed, cola_state* st, void* ws, size_t ws_bytes, void* stream) {
@@ -310,7 +310,7 @@ static int power_common(const cola_config* cfg, const cola_state* st, int32_t no
     if (rsd || std::fabs(a_out - a_node) > 1e-12 * a_node) {
         if (!(a_out > 0.0) || !state_ok(st, true)) return COLA_EINVAL;
         double* sp = reinterpret_cast<double*>(wsp(ws, kHdrSnap));
-        if ((rc = launch_snapshot_coeffs(cfg, a_node, a_out, sp, s))) return rc;
+        if ((rc = launch_snapshot_coeffs(cfg, a_node, a_out, sp, growth_ptr(ws), s))) return rc;
         snap = sp;
     }
     if ((rc = mark_dep_dirty(ws, s))) return rc;

@@ -469,7 +469,6 @@ __device__ __forceinline__ float2* fft_run_smem(const In& in, float2* a, float2*
 constexpr int kMaxSteps = 2048;
 constexpr int kTableCols = 12;
 constexpr size_t kHdrStatus = 0;          // int: latched device status
-constexpr size_t kHdrSigmaAmp = 64;       // double: P(k) amplitude A (sigma8 normalisation)
 constexpr size_t kHdrSnap = 128;          // 6 doubles: snapshot drift (dr, dD1, dD2), redshift-space (cv, c1, c2)
 constexpr size_t kHdrProbe = 512;         // 64 ints written by cola_checks_probe
 constexpr int kProbeInts = 64;
@@ -478,6 +477,7 @@ constexpr int kDepClean = 0x5a5a5a5a;     // (a byte pattern, so cudaMemsetAsync
 constexpr size_t kHdrFilter = 1024;       // radial filter basis table (<= 64 floats)
 constexpr size_t kHdrTable = 4096;        // kMaxSteps x kTableCols doubles
 constexpr size_t kHdrTwiddle = 262144;    // 3 slots of kMaxFft float2
+constexpr size_t kHdrGrowth = kHdrTwiddle + 3 * (size_t)kMaxFft * 8;  // scratch of the growth kernels
 constexpr size_t kHdrBytes = 524288;
 
 enum TwSlot { kTwMesh = 0, kTwLagr = 1, kTwScratch = 2 };
@@ -501,6 +501,7 @@ bool layout_for(const cola_config* cfg, Layout* L);
 inline char* wsp(void* ws, size_t off) { return static_cast<char*>(ws) + off; }
 inline int* status_ptr(void* ws) { return reinterpret_cast<int*>(wsp(ws, kHdrStatus)); }
 inline double* table_ptr(void* ws) { return reinterpret_cast<double*>(wsp(ws, kHdrTable)); }
+inline double* growth_ptr(void* ws) { return reinterpret_cast<double*>(wsp(ws, kHdrGrowth)); }
 inline float2* twiddle_ptr(void* ws, int slot) {
     return reinterpret_cast<float2*>(wsp(ws, kHdrTwiddle + (size_t)slot * kMaxFft * 8));
 }
@@ -668,8 +669,10 @@ size_t scan_sums_bytes(long long n);
 int step_node(const cola_config* cfg, cola_state* st, int32_t step, void* ws, size_t ws_bytes, cudaStream_t s,
               cudaEvent_t before_kick);
 
-int launch_tables(const cola_config* cfg, double* table, cudaStream_t s);
-int launch_snapshot_coeffs(const cola_config* cfg, double a_node, double a_out, double* snap, cudaStream_t s);
+// scratch: the workspace's growth scratch (kHdrGrowth)
+int launch_tables(const cola_config* cfg, double* table, double* scratch, cudaStream_t s);
+int launch_snapshot_coeffs(const cola_config* cfg, double a_node, double a_out, double* snap, double* scratch,
+                           cudaStream_t s);
 int launch_ic(const cola_config* cfg, uint64_t seed, cola_state st, void* ws, const Layout& L, cudaStream_t s);
 // p2, p4 (optional, both or neither): quadrupole and hexadecapole about the z axis
 int launch_power(const float2* mk, int ng, long long rs, double box, int flags, double* part, double* k, double* pk,
