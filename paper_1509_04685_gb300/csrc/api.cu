@@ -319,19 +319,19 @@ static int power_common(const cola_config* cfg, const cola_state* st, int32_t no
     const float2* tw = twiddles_for(ng_pk, cfg, ws, s, &rc);
     if (rc) return rc;
     const double ratio = (double)ng_pk / (double)cfg->nq;
-    // the region is shared with the step's bins: start from zero counts (the z pass clears them again)
+    // the region is shared with the step's bins: start from zero counts
     if (cudaMemsetAsync(dep, 0, (size_t)ng_pk * ng_pk * ng_pk * 8, s) != cudaSuccess) return COLA_ECUDA;
     if ((rc = launch_deposit_ex(st->d, st->v, st->psi1, st->psi2, dep, cfg->nq, ng_pk, cfg->box, snap,
                                 status_ptr(ws), s, rsd)))
         return rc;
     const long long Ppk = fft_pitch(ng_pk);
     if ((rc = fft_z_r2c(dep, mk, ng_pk, (float)(ratio * ratio * ratio / 1099511627776.0), tw, s, Ppk,
-                        (long long)ng_pk * ng_pk, FRow{ng_pk, 0, 1})))
+                        (long long)ng_pk * ng_pk, FRow{ng_pk, 0, 1}, false)))
         return rc;
     if ((rc = fft_strided(mk, ng_pk, 1, -1, tw, s))) return rc;
     if ((rc = fft_strided(mk, ng_pk, 0, -1, tw, s))) return rc;
-    return launch_power(mk, ng_pk, Ppk, cfg->box, flags, reinterpret_cast<double*>(wsp(ws, L.pk_part)), k, pk, nmodes,
-                        nbins, s, p2, p4);
+    return launch_power(mk, ng_pk, Ppk, cfg->box, flags, reinterpret_cast<double*>(wsp(ws, L.pk_part)),
+                        reinterpret_cast<float*>(dep), k, pk, nmodes, nbins, s, p2, p4);
 }
 
 extern "C" {

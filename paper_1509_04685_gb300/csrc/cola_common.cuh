@@ -593,8 +593,9 @@ int persistent_grid(size_t smem, int ntiles);
 int persistent_grid(size_t smem, int ntiles, int max_per_sm);
 // z passes: row r at base + r*rs (complex units), nrows rows
 // r2c: input row r = x n + y goes to output row frow(x, y, 0, fr) (fr = {n, 0, 1}: in place, same row)
+// dep: fixed-point counts to transform instead, cleared as they are read unless clear = false
 int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const float2* tw, cudaStream_t s,
-              long long rs, long long nrows, FRow fr);
+              long long rs, long long nrows, FRow fr, bool clear = true);
 int fft_z_c2r(float2* data, int n, const float2* tw, cudaStream_t s, float* out, long long opitch, float oscale,
               long long rs, long long nrows);
 // line passes: tile of outer index o starts at (o / o2n) s1 + (o % o2n) s2, element stride S
@@ -674,9 +675,10 @@ int launch_tables(const cola_config* cfg, double* table, double* scratch, cudaSt
 int launch_snapshot_coeffs(const cola_config* cfg, double a_node, double a_out, double* snap, double* scratch,
                            cudaStream_t s);
 int launch_ic(const cola_config* cfg, uint64_t seed, cola_state st, void* ws, const Layout& L, cudaStream_t s);
-// p2, p4 (optional, both or neither): quadrupole and hexadecapole about the z axis
-int launch_power(const float2* mk, int ng, long long rs, double box, int flags, double* part, double* k, double* pk,
-                 double* nmodes, int nbins, cudaStream_t s, double* p2 = nullptr, double* p4 = nullptr);
+// p2, p4 (optional, both or neither): quadrupole and hexadecapole about the z axis;
+// ctab: scratch of 8 ng^3 bytes (tables of the iterated Jing correction)
+int launch_power(const float2* mk, int ng, long long rs, double box, int flags, double* part, float* ctab, double* k,
+                 double* pk, double* nmodes, int nbins, cudaStream_t s, double* p2 = nullptr, double* p4 = nullptr);
 size_t power_partial_bytes(int nbins);
 
 // learned coarse-mesh correction (learned.cu)

@@ -51,12 +51,13 @@ int launch_twiddles(float2* tw, int n, cudaStream_t s) {
 // accessors for the z (row) passes.  Line l of a block is mesh row row0 + l.
 // ---------------------------------------------------------------------------
 // fixed-point CIC counts (2^40 per particle) -> delta = count*scale - 1, packed
-// as complex pairs; every count is cleared after it is read.
+// as complex pairs; every count is cleared after it is read (with `clear`).
 struct FixRowLoader {
     unsigned long long* dep;
     int n;
     long long row0, nrows;
     float scale;
+    bool clear;
     template <int R>
     __device__ __forceinline__ void load(int l, int i0, int di, float2* v) const {
         const long long row = row0 + l;
@@ -72,7 +73,7 @@ struct FixRowLoader {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             v[r] = make_float2((float)c[r].x * scale - 1.0f, (float)c[r].y * scale - 1.0f);
-            __stcs(p + i0 + r * di, make_ulonglong2(0ull, 0ull));
+            if (clear) __stcs(p + i0 + r * di, make_ulonglong2(0ull, 0ull));
         }
     }
 };
@@ -235,7 +236,8 @@ struct YZStore {
 // ---------------------------------------------------------------------------
 template <bool FIX>
 __global__ void k_fft_z_r2c(unsigned long long* __restrict__ dep, float2* out, int n, long long rs, long long nrows,
-                            int NR, float scale, FftPlan plan, const float2* __restrict__ tw, FastDiv m1div, FRow fr) {
+                            int NR, float scale, FftPlan plan, const float2* __restrict__ tw, FastDiv m1div, FRow fr,
+                            bool clear) {
     extern __shared__ float2 sm[];
     __shared__ long long obase[64];  // output row offsets of this block's lines
     const int M = n / 2;
@@ -250,7 +252,7 @@ __global__ void k_fft_z_r2c(unsigned long long* __restrict__ dep, float2* out, i
     const FftGeom g{NR, ls, 1, false, 0, 2};
     const float2* Z;
     if (FIX)
-        Z = fft_run_smem<-1, false>(FixRowLoader{dep, n, row0, nrows, scale}, sm, sb, plan, g, tw);
+        Z = fft_run_smem<-1, false>(FixRowLoader{dep, n, row0, nrows, scale, clear}, sm, sb, plan, g, tw);
     else
         Z = fft_run_smem<-1, false>(RowLoader{out, rs, row0, nrows}, sm, sb, plan, g, tw);
     for (int e = threadIdx.x; e < NR * (M + 1); e += blockDim.x) {
@@ -479,7 +481,7 @@ static int pass_threads(const FftPlan& plan, long lines) {
 }
 
 int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const float2* tw, cudaStream_t s,
-              long long rs, long long nrows, FRow fr) {
+              long long rs, long long nrows, FRow fr, bool clear) {
     FftPlan plan;
     if (!make_plan(n / 2, &plan)) return COLA_EUNSUPPORTED_SIZE;
     const int M = n / 2;
@@ -489,15 +491,15 @@ int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const fl
     const long long grid = (nrows + NR - 1) / NR;
     ProfScope ps(dep ? kKZr2cFix : kKZr2c, s);
     int rc = COLA_OK;
-    if (dep && launch_z_r2c_fix_static(dep, out, n, rs, nrows, scale, tw, fr, s, &rc)) return rc;
+    if (dep && launch_z_r2c_fix_static(dep, out, n, rs, nrows, scale, tw, fr, clear, s, &rc)) return rc;
     if (dep) {
         if (!set_smem((const void*)k_fft_z_r2c<true>, smem)) return COLA_ECUDA;
         k_fft_z_r2c<true><<<(unsigned)grid, T, smem, s>>>(dep, out, n, rs, nrows, NR, scale, plan, tw,
-                                                           make_fastdiv(M + 1), fr);
+                                                           make_fastdiv(M + 1), fr, clear);
     } else {
         if (!set_smem((const void*)k_fft_z_r2c<false>, smem)) return COLA_ECUDA;
         k_fft_z_r2c<false><<<(unsigned)grid, T, smem, s>>>(nullptr, out, n, rs, nrows, NR, 0.f, plan, tw,
-                                                            make_fastdiv(M + 1), fr);
+                                                            make_fastdiv(M + 1), fr, false);
     }
     return check_launch();
 }

@@ -8,6 +8,8 @@ namespace cola {
 // (n, B, threads) of every specialisation: B adjacent columns per tile, two
 // tile buffers of spad(n) B complex in shared memory
 #define COLA_STRIDED_SPECS(X) \
+    X(512, 16, 512) \
+    X(1024, 8, 512) \
     X(768, 16, 1024) \
     X(768, 8, 512) \
     X(1152, 8, 1024) \
@@ -26,16 +28,23 @@ namespace cola {
 
 // (n, B, threads) of the strided passes with two lines per thread; they take precedence
 #define COLA_STRIDED2_SPECS(X) \
+    X(512, 16, 256)             \
+    X(512, 8, 128)             \
+    X(1024, 8, 256)             \
     X(768, 16, 512)             \
     X(1152, 8, 384)             \
     X(1536, 8, 384)             \
     X(2304, 4, 384)
 #define COLA_YPSI2_SPECS(X) \
+    X(512, 16, 256)          \
+    X(1024, 8, 256)          \
     X(768, 16, 512)          \
     X(1152, 8, 384)          \
     X(1536, 8, 512)          \
     X(2304, 4, 384)
 #define COLA_XGREEN2_SPECS(X) \
+    X(512, 16, 256)          \
+    X(1024, 8, 256)          \
     X(768, 16, 384)            \
     X(1152, 8, 384)            \
     X(1536, 8, 384)            \
@@ -80,8 +89,8 @@ bool launch_x_green_static(float2* F, int n, int B, int nct, int ntiles, const f
 }
 
 // default column width of the specialised line passes of each size
-static const int kStaticTiles[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {288, 16}, {320, 16}, {384, 16}, {480, 16}, {768, 16}, {1152, 8}, {1536, 8}, {2304, 4}};
-static const int kStaticSpecs[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {256, 8}, {288, 16}, {320, 16}, {384, 16}, {384, 8}, {480, 16}, {480, 8}, {768, 16}, {768, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
+static const int kStaticTiles[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {288, 16}, {320, 16}, {384, 16}, {480, 16}, {512, 16}, {768, 16}, {1024, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
+static const int kStaticSpecs[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {256, 8}, {288, 16}, {320, 16}, {384, 16}, {384, 8}, {480, 16}, {480, 8}, {512, 16}, {512, 8}, {1024, 8}, {768, 16}, {768, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
 
 // default column width of the specialised fused x/Green pass of each size
 static const int kGreenTiles[][2] = {{768, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
@@ -108,6 +117,8 @@ bool static_tile_ok(int n, int B) {
 #define COLA_ZC2R_SPECS(X)   \
     X(256, 16, 256, 1)       \
     X(384, 8, 128, 1)        \
+    X(512, 8, 128, 2)        \
+    X(1024, 4, 128, 2)       \
     X(768, 8, 256, 2)        \
     X(1152, 4, 256, 2)       \
     X(1536, 4, 256, 2)       \
@@ -116,27 +127,32 @@ bool static_tile_ok(int n, int B) {
 #define COLA_ZR2C_SPECS(X)   \
     X(256, 16, 256, 1)       \
     X(384, 8, 128, 1)        \
+    X(512, 8, 128, 2)        \
+    X(1024, 4, 128, 2)       \
     X(768, 8, 256, 2)        \
     X(1152, 4, 256, 2)       \
     X(1536, 4, 256, 2)       \
     X(2304, 2, 256, 2)
 
 // (n, warps per block, blocks per SM) of the warp-row r2c of the fixed-point
-// counts; it takes precedence.  (At 1152 it was slower than the block tile,
+// counts; it takes precedence.  At 1024 it takes 2.11 ms against 4.32 ms for the
+// block tile (8 warps per SM fit there, 32 here), at 512 0.50 against 0.51 ms.  (At 1152 it was slower than the block tile,
 // 6.6 ms against 5.8 ms, and a warp-row plain c2r was slower at 2304, 74 ms
 // against 64 ms.)
 #define COLA_ZWARP_SPECS(X) \
+    X(512, 16, 2)           \
+    X(1024, 16, 2)          \
     X(2304, 16, 1)
 
 template <int N, int W, int MB>
 static int run_z_r2c_fix_w(unsigned long long* dep, float2* out, long long rs, long long nrows, float scale,
-                           const float2* tw, FRow fr, cudaStream_t s) {
+                           const float2* tw, FRow fr, bool clear, cudaStream_t s) {
     constexpr size_t smem = z_warp_smem<N, W>();
     static_assert((smem + 1024) * MB <= 227 * 1024, "MB blocks must fit");
     if (!set_smem((const void*)k_fft_z_r2c_fix_w<N, W, MB>, smem)) return COLA_ECUDA;
     const long long units = (nrows + W - 1) / W;
     k_fft_z_r2c_fix_w<N, W, MB><<<persistent_grid(smem, (int)(units < 0x7fffffff ? units : 0x7fffffff), MB),
-                                  32 * W, smem, s>>>(dep, out, rs, nrows, scale, tw, fr);
+                                  32 * W, smem, s>>>(dep, out, rs, nrows, scale, tw, fr, clear);
     return check_launch();
 }
 
@@ -154,17 +170,17 @@ bool launch_z_c2r_static(float2* data, int n, long long rs, long long nrows, con
 }
 
 bool launch_z_r2c_fix_static(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
-                             float scale, const float2* tw, FRow fr, cudaStream_t s, int* rc) {
+                             float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc) {
 #define COLA_CASE(NN, WW, MB)                                                               \
     if (n == NN && nrows == (long long)NN * NN) {                                          \
-        *rc = run_z_r2c_fix_w<NN, WW, MB>(dep, out, rs, nrows, scale, tw, fr, s);           \
+        *rc = run_z_r2c_fix_w<NN, WW, MB>(dep, out, rs, nrows, scale, tw, fr, clear, s);    \
         return true;                                                                        \
     }
     COLA_ZWARP_SPECS(COLA_CASE)
 #undef COLA_CASE
 #define COLA_CASE(NN, RR, TT, MB)                                                   \
     if (n == NN) {                                                                  \
-        *rc = run_z_r2c_fix<NN, RR, TT, MB>(dep, out, rs, nrows, scale, tw, fr, s); \
+        *rc = run_z_r2c_fix<NN, RR, TT, MB>(dep, out, rs, nrows, scale, tw, fr, clear, s); \
         return true;                                                                \
     }
     COLA_ZR2C_SPECS(COLA_CASE)

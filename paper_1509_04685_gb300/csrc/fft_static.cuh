@@ -1135,13 +1135,14 @@ template <int N>
 struct FixGlobal {
     unsigned long long* row;
     float scale;
+    bool clear;
     template <int R, int D>
     __device__ __forceinline__ void load(int, int i0, float2* v) const {
         ulonglong2* x = reinterpret_cast<ulonglong2*>(row);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const ulonglong2 c = __ldcs(x + i0 + r * D);
-            __stcs(x + i0 + r * D, make_ulonglong2(0ull, 0ull));
+            if (clear) __stcs(x + i0 + r * D, make_ulonglong2(0ull, 0ull));
             v[r] = make_float2((float)c.x * scale - 1.0f, (float)c.y * scale - 1.0f);
         }
     }
@@ -1162,7 +1163,7 @@ constexpr size_t z_warp_smem() {
 template <int N, int W, int MB>
 __global__ void __launch_bounds__(32 * W, MB) k_fft_z_r2c_fix_w(unsigned long long* __restrict__ dep, float2* out,
                                                                long long rs, long long nrows, float scale,
-                                                               const float2* __restrict__ tw, FRow fr) {
+                                                               const float2* __restrict__ tw, FRow fr, bool clear) {
     constexpr int M = N / 2;
     using Geo = WarpRow<M>;
     extern __shared__ float2 sm[];
@@ -1176,7 +1177,7 @@ __global__ void __launch_bounds__(32 * W, MB) k_fft_z_r2c_fix_w(unsigned long lo
     float2* Z = rows + w * Geo::LSTR;
     for (long long r = (long long)blockIdx.x * W + w; r < nrows; r += (long long)gridDim.x * W) {
         const int x = (int)(r / N), y = (int)(r - (long long)x * N);
-        sip_run<M, 32, Geo, -1, false, true>(FixGlobal<N>{dep + r * N, scale}, SSmem<Geo>{Z}, Z, tws, NoHook());
+        sip_run<M, 32, Geo, -1, false, true>(FixGlobal<N>{dep + r * N, scale, clear}, SSmem<Geo>{Z}, Z, tws, NoHook());
         // X[k] = E[k] + W^k O[k], E = (Z[k] + conj Z[M-k]) / 2, O = (Z[k] - conj Z[M-k]) / (2i)
         float2* orow = out + frow(x, y, 0, fr) * rs;
         for (int k = lane; k <= M; k += 32) {
@@ -1243,12 +1244,12 @@ __global__ void __launch_bounds__(T, MB) k_fft_z_c2r_s(float2* data, long long r
 }
 
 // forward r2c along z of the fixed-point CIC mesh (rows of N counts), which
-// is cleared as it is consumed; output row r = x n + y to frow(x, y, 0, fr)
-// (the runtime form is k_fft_z_r2c<true>)
+// is cleared as it is consumed (with `clear`); output row r = x n + y to
+// frow(x, y, 0, fr) (the runtime form is k_fft_z_r2c<true>)
 template <int N, int NR, int T, int MB>
 __global__ void __launch_bounds__(T, MB) k_fft_z_r2c_fix_s(unsigned long long* __restrict__ dep, float2* out,
                                                             long long rs, long long nrows, int ntiles, float scale,
-                                                            const float2* __restrict__ tw, FRow fr) {
+                                                            const float2* __restrict__ tw, FRow fr, bool clear) {
     constexpr int M = N / 2;
     using Geo = RowTile<M, NR>;
     constexpr int HN = N / 2;  // 16-byte chunks per count row
@@ -1278,7 +1279,7 @@ __global__ void __launch_bounds__(T, MB) k_fft_z_r2c_fix_s(unsigned long long* _
         __syncthreads();
         // the counts of this tile are in shared memory: clear them in the mesh
 #pragma unroll 4
-        for (int e = threadIdx.x; e < NR * HN; e += T) {
+        for (int e = clear ? threadIdx.x : NR * HN; e < NR * HN; e += T) {
             const int l = e / HN, c = (e - l * HN) * 2;
             if (row0 + l < nrows)
                 __stcs(reinterpret_cast<ulonglong2*>(dep + (row0 + l) * N + c), make_ulonglong2(0ull, 0ull));
@@ -1324,14 +1325,14 @@ inline int run_z_c2r(float2* data, long long rs, long long nrows, const float2* 
 
 template <int N, int NR, int T, int MB>
 inline int run_z_r2c_fix(unsigned long long* dep, float2* out, long long rs, long long nrows, float scale,
-                         const float2* tw, FRow fr, cudaStream_t s) {
+                         const float2* tw, FRow fr, bool clear, cudaStream_t s) {
     constexpr size_t smem = z_r2c_smem<N, NR, T>();
     static_assert((smem + 64 * NR + 1024) * MB <= 227 * 1024, "MB blocks must fit in shared memory");
     const long long nt = (nrows + NR - 1) / NR;
     if (nt > 0x7fffffff) return COLA_EUNSUPPORTED_SIZE;
     if (!set_smem((const void*)k_fft_z_r2c_fix_s<N, NR, T, MB>, smem)) return COLA_ECUDA;
     k_fft_z_r2c_fix_s<N, NR, T, MB><<<persistent_grid(smem, (int)nt, MB), T, smem, s>>>(dep, out, rs, nrows, (int)nt,
-                                                                                     scale, tw, fr);
+                                                                                     scale, tw, fr, clear);
     return check_launch();
 }
 
@@ -1346,7 +1347,7 @@ bool launch_x_green_static(float2* F, int n, int B, int nct, int ntiles, const f
 bool launch_z_c2r_static(float2* data, int n, long long rs, long long nrows, const float2* tw, cudaStream_t s,
                          int* rc);
 bool launch_z_r2c_fix_static(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
-                             float scale, const float2* tw, FRow fr, cudaStream_t s, int* rc);
+                             float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc);
 // default column width of the specialised line passes for n (0: none)
 int static_tile(int n);
 // whether (n, B) has specialised line passes
