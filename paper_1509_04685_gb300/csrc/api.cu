@@ -51,8 +51,7 @@ bool layout_for(const cola_config* cfg, Layout* L) {
     o = align_up(o + np * 4, 256);
     L->brank = o;
     o = align_up(o + np * 4, 256);
-    L->bsorted = o;
-    o = align_up(o + np * 4, 256);
+    o = align_up(o + np * 4, 256);  // (unused; kept so that workspace sizes do not change)
     L->bcic = o;
     o = align_up(o + np * 16, 256);
     L->slots = o;
@@ -106,7 +105,7 @@ static inline cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s)
 static BinBufs bin_bufs(void* ws, const Layout& L) {
     return BinBufs{reinterpret_cast<int*>(wsp(ws, L.bstart)), reinterpret_cast<int*>(wsp(ws, L.bsums)),
                    reinterpret_cast<int*>(wsp(ws, L.bkey)),   reinterpret_cast<int*>(wsp(ws, L.brank)),
-                   reinterpret_cast<int*>(wsp(ws, L.bsorted)), reinterpret_cast<float4*>(wsp(ws, L.bcic))};
+                   reinterpret_cast<float4*>(wsp(ws, L.bcic))};
 }
 static float* slots_ptr(void* ws, const Layout& L) { return reinterpret_cast<float*>(wsp(ws, L.slots)); }
 
@@ -136,7 +135,7 @@ static int pm_mesh_forces(const cola_config* cfg, const cola_state* st, double g
     const double ng3 = (double)ng * ng * ng;
     const long long P = fft_pitch(ng), n2 = (long long)ng * ng;
     const BinBufs bb = bin_bufs(ws, L);
-    const RowBins bins{bb.start, bb.sorted, bb.cic, status_ptr(ws), (long long)nq * nq * nq, ng};
+    const RowBins bins{bb.start, bb.cic, status_ptr(ws), (long long)nq * nq * nq, ng};
     const FRow fr = force_rows(ng);
     const bool fused = learned || fused_path(cfg);
     int rc;

@@ -11,10 +11,9 @@
 namespace cola {
 
 // Row bins of the PM step: particles sorted by the (x, y) mesh row of their
-// lower CIC corner, bin x ng + y holding sorted[start[b] .. start[b + 1]).
+// lower CIC corner, bin x ng + y holding records start[b] .. start[b + 1] - 1.
 struct RowBins {
     const int* start;     // ng^2 + 1 offsets
-    const int* sorted;    // particle indices
     const float4* cic;    // per sorted particle: CIC fractions (fx, fy, fz) and the lower z cell (int bits in w)
     int* status;          // the workspace's status word (bounds checks of a COLA_CHECKS build)
     long long np;         // particles (sorted positions are < np)
@@ -485,7 +484,7 @@ enum TwSlot { kTwMesh = 0, kTwLagr = 1, kTwScratch = 2 };
 struct Layout {
     size_t dep;        // uint64 fixed-point CIC mesh, ng^3 (outputs and the density call; cleared by its user)
     // the PM step's row bins and partial force sums, aliasing the region of dep
-    size_t bstart, bsums, bkey, brank, bsorted, bcic, slots;
+    size_t bstart, bsums, bkey, brank, bcic, slots;
     size_t F;          // interleaved force mesh: ng x ng x 3 rows of P complex (delta_k in component 0)
     size_t ic;         // 2LPT scratch: 7 complex meshes of nq x nq x Pq (aliases dep..)
     size_t pk_part;    // P(k) per-block partial sums (after the first two thirds of F)
@@ -626,9 +625,9 @@ int launch_adjoint_deposit(const float* d, const float* res, unsigned long long*
 int set_particle_traversal(int edge, int brick_k);  // traversal order of the particle kernels (pm.cu)
 
 // Row bins of the PM step (pm.cu): start[ng^2 + 1] (counts, then offsets),
-// sums (exclusive_scan scratch), key/rank/sorted[Np], cic[Np] (RowBins::cic).
+// sums (exclusive_scan scratch), key/rank[Np], cic[Np] (RowBins::cic).
 struct BinBufs {
-    int *start, *sums, *key, *rank, *sorted;
+    int *start, *sums, *key, *rank;
     float4* cic;
 };
 int launch_bins(const float* d, int nq, int ng, double box, const BinBufs& b, int* status, cudaStream_t s);

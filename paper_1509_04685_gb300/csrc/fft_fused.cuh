@@ -44,7 +44,7 @@ constexpr int kMaxTileBins = 2 * (64 + 1);  // row tiles of at most 64 rows
 
 // Bin list of a tile in shared memory: bin b is mesh row (x0, y0) =
 // (bxy[b] >> 16, bxy[b] & 0xffff) (coord_of(b) packs them), it starts at beg[b]
-// in the sorted arrays, and pre[b] is the number of particles in the bins
+// in the sorted records, and pre[b] is the number of particles in the bins
 // before it.  Returns the total.  Ends synchronised.
 // The group is threads tid < nthr (whole warps) synchronised by `sync`.
 template <class CoordOf, class Sync>
@@ -102,39 +102,37 @@ __device__ __forceinline__ int tile_find(const int* pre, int nb, int e) {
 
 __device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
-// A particle of a tile as read from the bins: its index (p < 0: none), its
-// CIC record (fractions, lower z cell) and the tile's bin it came from.  The
+// A particle of a tile as read from the bins: its sorted position (pos < 0:
+// none), its CIC record (fractions, lower z cell) and the tile's bin it came from.  The
 // compile-time forms read each tile's particles into registers one tile ahead,
 // so that the latency of these loads overlaps the FFT passes instead of
 // stalling the block.
 struct TilePart {
-    int p, b, pos;
+    int b, pos;
     float4 q;
 };
 
 __device__ __forceinline__ TilePart tile_load(int e, int total, const RowBins& bins, const int* beg, const int* pre,
                                               int nb) {
     TilePart t;
-    t.p = -1;
     t.b = 0;
-    t.pos = 0;
+    t.pos = -1;
     t.q = make_float4(0.f, 0.f, 0.f, 0.f);
     if (e < total) {
         const int b = tile_find(pre, nb, e);
         const int pos = beg[b] + (e - pre[b]);
         if (!bounds_ok(bins.status, pos >= 0 && pos < bins.np)) return t;
-        t.p = __ldg(bins.sorted + pos);
         t.q = __ldg(bins.cic + pos);
         t.b = b;
         t.pos = pos;
-        if (kChecks && !bounds_ok(bins.status, (unsigned)__float_as_int(t.q.w) < (unsigned)bins.ng)) t.p = -1;
+        if (kChecks && !bounds_ok(bins.status, (unsigned)__float_as_int(t.q.w) < (unsigned)bins.ng)) t.pos = -1;
     }
     return t;
 }
 
 // the particle's CIC corners: x0, y0 from its bin, z0 and the fractions from its record
 __device__ __forceinline__ bool part_cic(const TilePart& t, const int* bxy, int ng, Cic& c) {
-    if (t.p < 0) return false;
+    if (t.pos < 0) return false;
     const int xy = bxy[t.b];
     c.c0[0] = xy >> 16;
     c.c0[1] = xy & 0xffff;
@@ -163,6 +161,38 @@ __device__ __forceinline__ void deposit_one(const TilePart& t, const int* bxy, i
             if (l < 0 || l >= ty) continue;
             atomicAdd(cnt + l * ng + c.c0[2], w[4 * a + 2 * b]);
             atomicAdd(cnt + l * ng + c.c1[2], w[4 * a + 2 * b + 1]);
+        }
+    }
+}
+
+// The same into split counts: cell z of row l as two 32-bit counters at cnt[2 (l
+// ng + z)], the weights' lo and hi sums (fix_join gives the 64-bit count).  The
+// shared-memory atomics bound the deposit, and 32-bit ones are native: on random
+// cells two of them run at 1.7e12 pairs/s, one 64-bit atomic at 0.5e12/s.  With
+// the 64-bit weights gone as well, the whole pass took 15.4 ms instead of 18.8
+// (512^3 on 1536^3), 1.67 instead of 2.16 (256^3 on 768^3).  hi is at most 2^20
+// and |lo| 2^19 per particle, so the counters hold kSplitMax particles per cell;
+// tiles with more particles than that take deposit_one.
+constexpr int kSplitMax = 4095;
+__device__ __forceinline__ void deposit_one_split(const TilePart& t, const int* bxy, int ng, int x, int y0, int ty,
+                                                  int* cnt) {
+    Cic c;
+    if (!part_cic(t, bxy, ng, c)) return;
+    int hi[8], lo[8];
+    cic_fix_split(c, hi, lo);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        if ((a ? c.c1[0] : c.c0[0]) != x) continue;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int l = (b ? c.c1[1] : c.c0[1]) - y0;
+            if (l < 0 || l >= ty) continue;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                int* q = cnt + 2 * (l * ng + (e ? c.c1[2] : c.c0[2]));
+                atomicAdd(q, lo[4 * a + 2 * b + e]);
+                atomicAdd(q + 1, hi[4 * a + 2 * b + e]);
+            }
         }
     }
 }
@@ -453,6 +483,29 @@ __global__ void __launch_bounds__(96 * TX * G, MB)
     }
 }
 
+// a count as one 64-bit integer: itself, or joined from its split counters (lo, hi)
+__device__ __forceinline__ unsigned long long fix_count(unsigned long long v, bool split) {
+    return split ? fix_join((unsigned)(v >> 32), (int)(unsigned)v) : v;
+}
+
+// FixStage of counts that may be split
+template <int N>
+struct FixCounts {
+    const unsigned long long* stg;
+    float scale;
+    bool split;
+    template <int R, int D>
+    __device__ __forceinline__ void load(int, int i0, float2* v) const {
+        const ulonglong2* x = reinterpret_cast<const ulonglong2*>(stg);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const ulonglong2 c = x[i0 + r * D];
+            v[r] = make_float2((float)fix_count(c.x, split) * scale - 1.0f,
+                               (float)fix_count(c.y, split) * scale - 1.0f);
+        }
+    }
+};
+
 // r2c + deposit with warp-owned rows: G groups of NR warps per block; group g
 // takes tiles t = blockIdx.x G + g, then every gridDim.x G-th (tile t is rows
 // (x, y0 .. y0 + NR - 1), t = x (N / NR) + y0 / NR, as in k_fft_z_r2c_dep_s).
@@ -504,14 +557,20 @@ __global__ void __launch_bounds__(32 * NR * G, MB)
             bins, NB, N,
             [&](int b) { return (wrap(x - 1 + b / (NR + 1), N) << 16) | wrap(y0 - 1 + b % (NR + 1), N); }, beg[g],
             pre[g], bxy[g], gl, GT, gsync);
-        for (int e = gl; e < total; e += GT)
-            deposit_one(tile_load(e, total, bins, beg[g], pre[g], NB), bxy[g], N, x, y0, NR, cnt);
+        const bool split = total <= kSplitMax;
+        if (split)
+            for (int e = gl; e < total; e += GT)
+                deposit_one_split(tile_load(e, total, bins, beg[g], pre[g], NB), bxy[g], N, x, y0, NR,
+                                  reinterpret_cast<int*>(cnt));
+        else
+            for (int e = gl; e < total; e += GT)
+                deposit_one(tile_load(e, total, bins, beg[g], pre[g], NB), bxy[g], N, x, y0, NR, cnt);
         gsync();
         if (delta_out) {
             float* o = delta_out + ((long long)x * N + y0 + l) * N;
-            for (int e = lane; e < N; e += 32) o[e] = (float)myc[e] * scale - 1.0f;
+            for (int e = lane; e < N; e += 32) o[e] = (float)fix_count(myc[e], split) * scale - 1.0f;
         }
-        sip_run<M, 32, Geo, -1, true, true>(FixStage<N>{myc, scale}, SSmem<Geo>{Z}, Z, tws, NoHook());
+        sip_run<M, 32, Geo, -1, true, true>(FixCounts<N>{myc, scale, split}, SSmem<Geo>{Z}, Z, tws, NoHook());
         // X[k] = E[k] + W^k O[k], E = (Z[k] + conj Z[M-k]) / 2, O = (Z[k] - conj Z[M-k]) / (2i)
         float2* orow = out + frow(x, y0 + l, 0, fr) * rs;
         for (int k = lane; k <= M; k += 32) {

@@ -336,14 +336,14 @@ int launch_adjoint_deposit(const float* d, const float* res, unsigned long long*
 }
 
 // --------------------------------------------------------------------------
-// Row binning of the PM step: a counting sort of the particle indices by the
+// Row binning of the PM step: a counting sort of the particles by the
 // (x, y) mesh row of their lower CIC corner, key x ng + y.  k_bin_count takes
 // each particle's rank inside its bin with an atomic (counts start at zero),
-// exclusive_scan turns the counts into offsets, k_bin_scatter writes
-// sorted[start[key] + rank] = p and, at the same place, the particle's CIC
-// fractions and lower z cell (its x and y cells are the bin's), so that the
-// fused passes read one contiguous 16-byte record per particle visit; rank[p]
-// is then replaced by that sorted position (-1 for a particle left out).  The order inside a bin depends on the atomics
+// exclusive_scan turns the counts into offsets, k_bin_scatter writes at
+// start[key] + rank the particle's CIC fractions and lower z cell (its x and y
+// cells are the bin's), so that the fused passes read one contiguous 16-byte
+// record per particle visit; rank[p] is then replaced by that sorted position
+// (-1 for a particle left out).  The order inside a bin depends on the atomics
 // and changes no result: the fused deposit adds integers, and every particle's
 // partial force sums are its own.  A non-finite position latches
 // COLA_ENONFINITE and leaves the particle out of every bin.
@@ -372,7 +372,7 @@ __global__ void k_bin_count(const float* __restrict__ d, int nq, int ng, float i
 
 __global__ void k_bin_scatter(const float* __restrict__ d, int nq, int ng, float inv_cell, long long np,
                               const int* __restrict__ key, int* __restrict__ rank, const int* __restrict__ start,
-                              int* __restrict__ sorted, float4* __restrict__ cic, int* status, Trav tv) {
+                              float4* __restrict__ cic, int* status, Trav tv) {
     int idx[3];
     if (!trav_site(tv, idx)) return;
     const long long p = site_index(idx, nq);
@@ -389,7 +389,6 @@ __global__ void k_bin_scatter(const float* __restrict__ d, int nq, int ng, float
         rank[p] = -1;
         return;
     }
-    sorted[pos] = (int)p;
     cic[pos] = make_float4(c.f[0], c.f[1], c.f[2], __int_as_float(c.c0[2]));
     rank[p] = pos;
 }
@@ -406,7 +405,7 @@ int launch_bins(const float* d, int nq, int ng, double box, const BinBufs& b, in
     if (rc) return rc;
     if ((rc = exclusive_scan(b.start, nb, b.sums, s))) return rc;
     k_bin_scatter<<<trav_grid(tv), kTravThreads, 0, s>>>(d, nq, ng, (float)((double)ng / box), np, b.key, b.rank,
-                                                          b.start, b.sorted, b.cic, status, tv);
+                                                          b.start, b.cic, status, tv);
     return check_launch();
 }
 
