@@ -1348,6 +1348,10 @@ bool launch_z_c2r_static(float2* data, int n, long long rs, long long nrows, con
                          int* rc);
 bool launch_z_r2c_fix_static(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
                              float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc);
+bool launch_z_c2r_static_small(float2* data, int n, long long rs, long long nrows, const float2* tw, cudaStream_t s,
+                               int* rc);
+bool launch_z_r2c_fix_static_small(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
+                                   float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc);
 // default column width of the specialised line passes for n (0: none)
 int static_tile(int n);
 // whether (n, B) has specialised line passes
