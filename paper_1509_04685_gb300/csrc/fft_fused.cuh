@@ -272,6 +272,29 @@ constexpr size_t z_r2c_dep_smem() {
 constexpr int kDepAhead = 3;
 constexpr int kGatherAhead = 2;
 
+// a count as one 64-bit integer: itself, or joined from its split counters (lo, hi)
+__device__ __forceinline__ unsigned long long fix_count(unsigned long long v, bool split) {
+    return split ? fix_join((unsigned)(v >> 32), (int)(unsigned)v) : v;
+}
+
+// FixStage of counts that may be split
+template <int N>
+struct FixCounts {
+    const unsigned long long* stg;
+    float scale;
+    bool split;
+    template <int R, int D>
+    __device__ __forceinline__ void load(int l, int i0, float2* v) const {
+        const ulonglong2* x = reinterpret_cast<const ulonglong2*>(stg + (size_t)l * N);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const ulonglong2 c = x[i0 + r * D];
+            v[r] = make_float2((float)fix_count(c.x, split) * scale - 1.0f,
+                               (float)fix_count(c.y, split) * scale - 1.0f);
+        }
+    }
+};
+
 // r2c + deposit: tiles of TY = NR rows of one x, t = x (N / NR) + y0 / NR.
 // Per tile: clear the counts, deposit the particles read during the previous
 // tile's transform, list the next tile's bins and read its particles, then the
@@ -318,10 +341,19 @@ __global__ void __launch_bounds__(T, MB)
         for (int e = threadIdx.x; e < NR * N / 2; e += T) c2[e] = make_ulonglong2(0ull, 0ull);
         if (threadIdx.x < NR) obase[threadIdx.x] = frow(x, y0 + threadIdx.x, 0, fr) * rs;
         __syncthreads();
+        const bool split = total <= kSplitMax;
+        if (split) {
+            int* c = reinterpret_cast<int*>(cnt);
 #pragma unroll
-        for (int k = 0; k < kDepAhead; ++k) deposit_one(ahead[k], bxy, N, x, y0, NR, cnt);
-        for (int e = threadIdx.x + kDepAhead * T; e < total; e += T)
-            deposit_one(tile_load(e, total, bins, beg, pre, NB), bxy, N, x, y0, NR, cnt);
+            for (int k = 0; k < kDepAhead; ++k) deposit_one_split(ahead[k], bxy, N, x, y0, NR, c);
+            for (int e = threadIdx.x + kDepAhead * T; e < total; e += T)
+                deposit_one_split(tile_load(e, total, bins, beg, pre, NB), bxy, N, x, y0, NR, c);
+        } else {
+#pragma unroll
+            for (int k = 0; k < kDepAhead; ++k) deposit_one(ahead[k], bxy, N, x, y0, NR, cnt);
+            for (int e = threadIdx.x + kDepAhead * T; e < total; e += T)
+                deposit_one(tile_load(e, total, bins, beg, pre, NB), bxy, N, x, y0, NR, cnt);
+        }
         __syncthreads();
         const int tn = t + gridDim.x;
         if (tn < ntiles) {
@@ -331,9 +363,9 @@ __global__ void __launch_bounds__(T, MB)
         }
         if (delta_out) {
             float* o = delta_out + ((long long)x * N + y0) * N;
-            for (int e = threadIdx.x; e < NR * N; e += T) o[e] = (float)cnt[e] * scale - 1.0f;
+            for (int e = threadIdx.x; e < NR * N; e += T) o[e] = (float)fix_count(cnt[e], split) * scale - 1.0f;
         }
-        const float2* Z = srun_smem<M, T, Geo, -1>(FixStage<N>{cnt, scale}, A, Bf, tws, NoHook());
+        const float2* Z = srun_smem<M, T, Geo, -1>(FixCounts<N>{cnt, scale, split}, A, Bf, tws, NoHook());
         // X[k] = E[k] + W^k O[k], E = (Z[k] + conj Z[M-k]) / 2, O = (Z[k] - conj Z[M-k]) / (2i)
 #pragma unroll 2
         for (int e = threadIdx.x; e < NR * (M + 1); e += T) {
@@ -482,29 +514,6 @@ __global__ void __launch_bounds__(96 * TX * G, MB)
         gsync();  // the rows and the bin list are reused by the group's next tile
     }
 }
-
-// a count as one 64-bit integer: itself, or joined from its split counters (lo, hi)
-__device__ __forceinline__ unsigned long long fix_count(unsigned long long v, bool split) {
-    return split ? fix_join((unsigned)(v >> 32), (int)(unsigned)v) : v;
-}
-
-// FixStage of counts that may be split
-template <int N>
-struct FixCounts {
-    const unsigned long long* stg;
-    float scale;
-    bool split;
-    template <int R, int D>
-    __device__ __forceinline__ void load(int, int i0, float2* v) const {
-        const ulonglong2* x = reinterpret_cast<const ulonglong2*>(stg);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const ulonglong2 c = x[i0 + r * D];
-            v[r] = make_float2((float)fix_count(c.x, split) * scale - 1.0f,
-                               (float)fix_count(c.y, split) * scale - 1.0f);
-        }
-    }
-};
 
 // r2c + deposit with warp-owned rows: G groups of NR warps per block; group g
 // takes tiles t = blockIdx.x G + g, then every gridDim.x G-th (tile t is rows

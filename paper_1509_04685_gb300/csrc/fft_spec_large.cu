@@ -192,10 +192,18 @@ bool launch_z_r2c_fix_static(unsigned long long* dep, float2* out, int n, long l
 
 
 
-// (n, rows per tile, threads, blocks per SM) of the fused r2c + deposit pass
+// (n, rows per tile, threads, blocks per SM) of the fused r2c + deposit pass.  The
+// meshes below 256 are those of the learned net, which takes this pass at any
+// size: at 128 the runtime form took 389 us, tiles of 32 rows (512 tiles for 456
+// resident blocks) 305, of 16 rows 203.
 #define COLA_ZR2CD_SPECS(X) \
-    X(256, 16, 256, 1)      \
-    X(384, 8, 128, 1)       \
+    X(64, 16, 128, 6)       \
+    X(96, 16, 128, 6)       \
+    X(128, 16, 128, 5)      \
+    X(160, 16, 128, 4)      \
+    X(192, 16, 128, 4)      \
+    X(256, 16, 256, 3)      \
+    X(384, 8, 128, 3)       \
     X(768, 8, 256, 2)       \
     X(1152, 4, 256, 2)      \
     X(1536, 4, 256, 2)      \

@@ -31,6 +31,27 @@ __device__ __forceinline__ void mma_bf16_16816(float* c, const unsigned* a, cons
 
 __device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
+// Voxel rows in shared memory: 16 channels = two 16-byte halves, half h of row v at
+// chunk 2 v + (h ^ bit 2 of v), so that the eight rows an 8 x 8 matrix load takes
+// (any eight consecutive voxels) lie in different banks.
+__device__ __forceinline__ int chunk_of(int v, int h) { return 2 * v + (h ^ ((v >> 2) & 1)); }
+
+__device__ __forceinline__ void ldmatrix_x4(unsigned* r, const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(unsigned* r, const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldmatrix_x2(unsigned* r, const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+
 enum ConvEpi { kEpiBiasRelu = 0, kEpiAddForce = 1, kEpiMask = 2 };
 
 // Forward stencil conv (also the data gradient, with flipped/transposed
@@ -39,6 +60,10 @@ enum ConvEpi { kEpiBiasRelu = 0, kEpiAddForce = 1, kEpiMask = 2 };
 //   kEpiBiasRelu: out[v][co] = bf16(relu(acc + bias))
 //   kEpiAddForce: F[((x N + y) 3 + c) P2 + z] += scale (acc + bias), c < 3 (force-mesh real view)
 //   kEpiMask:     out[v][co] = bf16(acc * (mask[v][co] > 0))
+// Bound by shared-memory loads: a warp takes the four z-rows of its y at once, so
+// the weights of a tap are loaded once for the four, and fragments come by matrix
+// loads (16 -> 16 channels at 128^3: 217 us with 32-bit fragment loads per row and
+// tap, now 105).
 template <int NT, int EPI>
 __global__ void __launch_bounds__(kConvWarps * 32) k_conv(const bf16* __restrict__ x, const bf16* __restrict__ w,
                                                           const float* __restrict__ bias, int N, bf16* out,
@@ -60,32 +85,43 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(const bf16* __restrict
         const int hv = e >> 1;
         const int hz = hv % kHz, hy = (hv / kHz) % kHy, hx = hv / (kHz * kHy);
         const long long v = ((long long)wrap(x0 + hx, N) * N + wrap(y0 + hy, N)) * N + wrap(z0 + hz, N);
-        reinterpret_cast<uint4*>(sx)[e] = reinterpret_cast<const uint4*>(x + v * CIN)[half];
+        reinterpret_cast<uint4*>(sx)[chunk_of(hv, half)] = reinterpret_cast<const uint4*>(x + v * CIN)[half];
     }
     for (int e = threadIdx.x; e < 27 * COUT * CIN / 8; e += blockDim.x)
-        reinterpret_cast<uint4*>(sw)[e] = reinterpret_cast<const uint4*>(w)[e];
+        reinterpret_cast<uint4*>(sw)[chunk_of(e >> 1, e & 1)] = reinterpret_cast<const uint4*>(w)[e];
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tg = lane & 3;
-    for (int tile = warp; tile < kBx * kBy; tile += kConvWarps) {
-        const int lx = tile / kBy, ly = tile % kBy;  // one z-row of 16 voxels
-        float acc[NT][4];
+    static_assert(kBy == kConvWarps, "warp = y row of the brick");
+    const int ly = warp;
+    const int arow = (lane & 7) + (lane & 8), ahalf = lane >> 4;                        // A: rows 0-7, 8-15; k 0-7, 8-15
+    const int brow = (lane & 7) + (NT == 2 ? (lane >> 4) * 8 : 0), bhalf = (lane >> 3) & 1;  // B: n tiles of k 0-7, 8-15
+    float accs[kBx][NT][4];
 #pragma unroll
-        for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+    for (int i = 0; i < kBx; ++i)
+#pragma unroll
+        for (int n = 0; n < NT; ++n) accs[i][n][0] = accs[i][n][1] = accs[i][n][2] = accs[i][n][3] = 0.f;
 #pragma unroll 3
-        for (int t = 0; t < 27; ++t) {
-            const int tx = t / 9, ty = (t / 3) % 3, tz = t % 3;
-            const int hbase = ((lx + tx) * kHy + (ly + ty)) * kHz + tz;
-            const unsigned* r0 = reinterpret_cast<const unsigned*>(sx + (hbase + g) * CIN);
-            const unsigned* r1 = reinterpret_cast<const unsigned*>(sx + (hbase + g + 8) * CIN);
-            unsigned a[4] = {r0[tg], r1[tg], r0[tg + 4], r1[tg + 4]};
+    for (int t = 0; t < 27; ++t) {
+        const int tx = t / 9, ty = (t / 3) % 3, tz = t % 3;
+        unsigned bb[4];
+        const bf16* wp = sw + chunk_of(t * COUT + brow, bhalf) * 8;
+        if (NT == 2)
+            ldmatrix_x4(bb, wp);
+        else
+            ldmatrix_x2(bb, wp);
 #pragma unroll
-            for (int n = 0; n < NT; ++n) {
-                const unsigned* wb = reinterpret_cast<const unsigned*>(sw + (t * COUT + n * 8 + g) * CIN);
-                unsigned bb[2] = {wb[tg], wb[tg + 4]};
-                mma_bf16_16816(acc[n], a, bb);
-            }
+        for (int i = 0; i < kBx; ++i) {
+            const int hbase = ((i + tx) * kHy + (ly + ty)) * kHz + tz;
+            unsigned a[4];
+            ldmatrix_x4(a, sx + chunk_of(hbase + arow, ahalf) * 8);
+#pragma unroll
+            for (int n = 0; n < NT; ++n) mma_bf16_16816(accs[i][n], a, bb + 2 * n);
         }
+    }
+#pragma unroll
+    for (int lx = 0; lx < kBx; ++lx) {
+        float(&acc)[NT][4] = accs[lx];
         // epilogue: rows g and g+8 of the tile are voxels z = g, g+8; columns co = 2 tg, 2 tg + 1
         const int vx = bx * kBx + lx, vy = by * kBy + ly;
 #pragma unroll
@@ -120,7 +156,9 @@ __global__ void __launch_bounds__(kConvWarps * 32) k_conv(const bf16* __restrict
 // (16 channels each; padded channels are zero).  A = dy^T (co x voxels),
 // B = shifted x (voxels x ci); each warp owns three taps, blocks are
 // persistent over bricks and write one partial per block (fixed-order
-// reduction afterwards keeps the result deterministic).
+// reduction afterwards keeps the result deterministic).  Fragments come by
+// transposing matrix loads (with 16-bit element loads: 316 us per layer at 128^3,
+// now 151).
 constexpr size_t kDwSmem = (size_t)(kHx * kHy * kHz + kBx * kBy * kBz) * 16 * sizeof(bf16);
 
 __global__ void __launch_bounds__(288) k_conv_dw(const bf16* __restrict__ x, const bf16* __restrict__ dy, int N,
@@ -152,50 +190,33 @@ __global__ void __launch_bounds__(288) k_conv_dw(const bf16* __restrict__ x, con
             const int hv = e >> 1;
             const int hz = hv % kHz, hy = (hv / kHz) % kHy, hx = hv / (kHz * kHy);
             const long long v = ((long long)wrap(x0 + hx, N) * N + wrap(y0 + hy, N)) * N + wrap(z0 + hz, N);
-            reinterpret_cast<uint4*>(sx)[e] = reinterpret_cast<const uint4*>(x + v * CIN)[half];
+            reinterpret_cast<uint4*>(sx)[chunk_of(hv, half)] = reinterpret_cast<const uint4*>(x + v * CIN)[half];
         }
         for (int e = threadIdx.x; e < kBx * kBy * kBz * COUT / 8; e += blockDim.x) {
             const int per = COUT / 8;
             const int bv = e / per, part8 = e % per;
             const int lz = bv % kBz, ly = (bv / kBz) % kBy, lx = bv / (kBz * kBy);
             const long long v = ((long long)(bx * kBx + lx) * N + (by * kBy + ly)) * N + (bz * kBz + lz);
-            reinterpret_cast<uint4*>(sd)[e] = reinterpret_cast<const uint4*>(dy + v * COUT)[part8];
+            reinterpret_cast<uint4*>(sd)[chunk_of(bv, part8)] = reinterpret_cast<const uint4*>(dy + v * COUT)[part8];
         }
         __syncthreads();
         if (warp < 9) {
             // K loop over the brick's voxels, 16 at a time (one z-row)
             for (int row = 0; row < kBx * kBy; ++row) {
                 const int lx = row / kBy, ly = row % kBy;
-                // A fragment: A[co][v], co = g / g+8, v = 2tg, 2tg+1 / +8, +9 (z offsets in the row)
+                // A fragment: A[co][v] from rows [v][co], transposed 8 x 8 blocks (v 0-7, 8-15; co 0-7, 8-15)
                 unsigned a[4];
-                {
-                    const bf16* d0 = sd + ((lx * kBy + ly) * kBz) * COUT;
-                    auto pk = [&](int co, int vz) -> unsigned {
-                        const bf16 lo = co < COUT ? d0[vz * COUT + co] : __float2bfloat16(0.f);
-                        const bf16 hi = co < COUT ? d0[(vz + 1) * COUT + co] : __float2bfloat16(0.f);
-                        return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
-                    };
-                    a[0] = pk(g, 2 * tg);
-                    a[1] = pk(g + 8, 2 * tg);
-                    a[2] = pk(g, 2 * tg + 8);
-                    a[3] = pk(g + 8, 2 * tg + 8);
-                }
+                ldmatrix_x4_trans(a, sd + chunk_of(row * kBz + (lane & 7) + (lane >> 4) * 8, (lane >> 3) & 1) * 8);
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
                     const int t = warp * 3 + q;
                     const int tx = t / 9, ty = (t / 3) % 3, tz = t % 3;
-                    const bf16* xs = sx + (((lx + tx) * kHy + (ly + ty)) * kHz + tz) * CIN;
-#pragma unroll
-                    for (int n = 0; n < 2; ++n) {
-                        // B fragment: B[v][ci], v = 2tg, 2tg+1 (reg 0) / +8, +9 (reg 1), ci = n*8 + g
-                        const int ci = n * 8 + g;
-                        auto pb = [&](int vz) -> unsigned {
-                            return (unsigned)__bfloat16_as_ushort(xs[vz * CIN + ci]) |
-                                   ((unsigned)__bfloat16_as_ushort(xs[(vz + 1) * CIN + ci]) << 16);
-                        };
-                        unsigned bb[2] = {pb(2 * tg), pb(2 * tg + 8)};
-                        mma_bf16_16816(acc[q][n], a, bb);
-                    }
+                    const int hv = ((lx + tx) * kHy + (ly + ty)) * kHz + tz;
+                    // B fragments of both ci tiles: B[v][ci] from rows [v][ci], transposed blocks
+                    unsigned bb[4];
+                    ldmatrix_x4_trans(bb, sx + chunk_of(hv + (lane & 7) + (lane & 8), lane >> 4) * 8);
+                    mma_bf16_16816(acc[q][0], a, bb);
+                    mma_bf16_16816(acc[q][1], a, bb + 2);
                 }
             }
         }
@@ -221,30 +242,69 @@ __global__ void __launch_bounds__(288) k_conv_dw(const bf16* __restrict__ x, con
     }
 }
 
-// fixed-order sum of per-block partials: out[i] = sum_b part[b][i]
-__global__ void k_sum_partials(const float* __restrict__ part, int nblocks, int len, float* out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= len) return;
+// Fixed-order sums of the per-block partials [block][27][16][16] of a weight
+// gradient, written in the master layout [co][ci][27]: 32 elements per block of
+// 32 x 16 threads, thread row y adding partials y, y + 16, ...
+constexpr int kSumRows = 16;
+__global__ void __launch_bounds__(32 * kSumRows) k_dw_finish(const float* __restrict__ part, int nblocks, int co_n,
+                                                             int ci_n, float* __restrict__ out) {
+    __shared__ float red[kSumRows][32];
+    const int i = blockIdx.x * 32 + threadIdx.x;  // (t 16 + co) 16 + ci
     float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * len + i];
-    out[i] = s;
+    for (int b = threadIdx.y; b < nblocks; b += kSumRows) s += part[(size_t)b * 27 * 256 + i];
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y) return;
+    for (int y = 1; y < kSumRows; ++y) s += red[y][threadIdx.x];
+    const int ci = i % 16, co = (i / 16) % 16, t = i / 256;
+    if (co < co_n && ci < ci_n) out[(co * ci_n + ci) * 27 + t] = s;
 }
 
-// bias gradient partials: db[co] = sum_v dy[v][co] (dy with 16 channels)
-__global__ void k_bias_grad(const bf16* __restrict__ dy, long long nv, int cout, float* __restrict__ part) {
-    __shared__ float red[256][16];
-    float s[16];
-    for (int c = 0; c < 16; ++c) s[c] = 0.f;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += (long long)gridDim.x * blockDim.x)
-        for (int c = 0; c < cout; ++c) s[c] += __bfloat162float(dy[v * 16 + c]);
-    for (int c = 0; c < 16; ++c) red[threadIdx.x][c] = s[c];
+// bias gradient: out[co] = sum of part[block][co]
+__global__ void __launch_bounds__(512) k_db_finish(const float* __restrict__ part, int nblocks, int cout, float* out) {
+    __shared__ float red[32][16];
+    const int c = threadIdx.x & 15, y = threadIdx.x >> 4;
+    float s = 0.f;
+    if (c < cout)
+        for (int b = y; b < nblocks; b += 32) s += part[(size_t)b * cout + c];
+    red[y][c] = s;
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st)
-            for (int c = 0; c < 16; ++c) red[threadIdx.x][c] += red[threadIdx.x + st][c];
-        __syncthreads();
+    if (y || c >= cout) return;
+    for (int q = 1; q < 32; ++q) s += red[q][c];
+    out[c] = s;
+}
+
+// bias gradient partials: db[co] = sum_v dy[v][co] (dy with 16 channels); a
+// thread adds one 8-channel half of every 128th voxel row of its block's share
+__global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ dy, long long nv, int cout,
+                                                   float* __restrict__ part) {
+    __shared__ float red[8][16];
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const int half = threadIdx.x & 1;
+    if (8 * half < cout)
+        for (long long v = (long long)blockIdx.x * 128 + (threadIdx.x >> 1); v < nv; v += (long long)gridDim.x * 128) {
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(dy + v * 16) + half);
+            const unsigned w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                s[2 * c] += __uint_as_float(w[c] << 16);
+                s[2 * c + 1] += __uint_as_float(w[c] & 0xffff0000u);
+            }
+        }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+#pragma unroll
+        for (int o = 2; o < 32; o <<= 1) s[c] += __shfl_xor_sync(0xffffffffu, s[c], o);
     }
-    if (threadIdx.x < cout) part[blockIdx.x * cout + threadIdx.x] = red[0][threadIdx.x];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (lane < 2)
+        for (int c = 0; c < 8; ++c) red[w][8 * lane + c] = s[c];
+    __syncthreads();
+    if (threadIdx.x < cout) {
+        float t = 0.f;
+        for (int q = 0; q < 8; ++q) t += red[q][threadIdx.x];
+        part[blockIdx.x * cout + threadIdx.x] = t;
+    }
 }
 
 // network input: channels (delta, F_x/g, F_y/g, F_z/g, 0...) as bf16 [v][16]
@@ -271,14 +331,19 @@ __global__ void k_pack_input(const float* __restrict__ delta, const float* __res
     }
 }
 
-// upstream gradient of the last layer: dy[v][c] = g * dL/dF_c(v) (c < 3), 0 above
-__global__ void k_pack_grad(const float* __restrict__ dF, int N, float gsc, bf16* __restrict__ dy) {
+// upstream gradient of the last layer: dy[v][c] = g * dL/dF_c(v) (c < 3), 0 above,
+// dL/dF_c = fix3 scale from the fixed-point adjoint deposit
+__global__ void k_pack_grad(const unsigned long long* __restrict__ fix3, int N, float scale, float gsc,
+                            bf16* __restrict__ dy) {
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long n3 = (long long)N * N * N;
     if (v >= n3) return;
+    float f[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f[c] = __fmul_rn((float)(long long)fix3[c * n3 + v], scale);
     __nv_bfloat162 h[8];
-    h[0] = __floats2bfloat162_rn(gsc * dF[v], gsc * dF[n3 + v]);
-    h[1] = __floats2bfloat162_rn(gsc * dF[2 * n3 + v], 0.f);
+    h[0] = __floats2bfloat162_rn(gsc * f[0], gsc * f[1]);
+    h[1] = __floats2bfloat162_rn(gsc * f[2], 0.f);
     for (int q = 2; q < 8; ++q) h[q] = __floats2bfloat162_rn(0.f, 0.f);
     reinterpret_cast<uint4*>(dy + v * 16)[0] = reinterpret_cast<uint4*>(h)[0];
     reinterpret_cast<uint4*>(dy + v * 16)[1] = reinterpret_cast<uint4*>(h)[1];
@@ -325,9 +390,12 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ gsum, fl
 // particle side of the training loss
 // L = 1/(2 Np) sum_p |F_pred(p) - F_target(p)|^2; residual r = F_pred - F_target
 // --------------------------------------------------------------------------
-__global__ void k_residual(const float* __restrict__ pred, const float* __restrict__ target, float* __restrict__ res,
-                           long long n3p, double* __restrict__ part) {
-    __shared__ double red[256];
+constexpr int kLossThreads = 1024;
+__global__ void __launch_bounds__(kLossThreads) k_residual(const float* __restrict__ pred,
+                                                           const float* __restrict__ target,
+                                                           float* __restrict__ res, long long n3p,
+                                                           double* __restrict__ part) {
+    __shared__ double red[kLossThreads];
     double acc = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3p; i += (long long)gridDim.x * blockDim.x) {
         const float r = pred[i] - target[i];
@@ -343,11 +411,16 @@ __global__ void k_residual(const float* __restrict__ pred, const float* __restri
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-__global__ void k_sum_double(const double* __restrict__ part, int n, double scale, double* out) {
-    if (threadIdx.x || blockIdx.x) return;
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
-    *out = s * scale;
+// n <= 512
+__global__ void __launch_bounds__(512) k_sum_double(const double* __restrict__ part, int n, double scale, double* out) {
+    __shared__ double red[512];
+    red[threadIdx.x] = threadIdx.x < n ? part[threadIdx.x] : 0.0;
+    __syncthreads();
+    for (int st = 256; st > 0; st >>= 1) {
+        if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *out = red[0] * scale;
 }
 
 // Normal equations of the k-space filter fit: with basis force columns
@@ -422,9 +495,8 @@ constexpr int kPf1 = 0, kPf2 = 6912, kPf3 = 13824, kPd2 = 17280, kPd3 = 24192;
 struct LearnedBufs {
     float* delta;
     bf16 *x0, *h1, *h2, *g1, *g2;
-    float* dF;
     unsigned long long* fix3;
-    float *pred, *res, *dwpart, *dwsum, *bpart;
+    float *pred, *res, *dwpart, *bpart;
     double* lpart;
 };
 
@@ -452,12 +524,12 @@ static LearnedBufs learned_bufs(char* base, int ng, int nq) {
     B.h2 = (bf16*)take(32 * n3);
     B.g1 = (bf16*)take(32 * n3);
     B.g2 = (bf16*)take(32 * n3);
-    B.dF = (float*)take(12 * n3);
+    take(12 * n3);  // (unused; kept so that workspace sizes do not change)
     B.fix3 = (unsigned long long*)take(24 * n3);
     B.pred = (float*)take(12 * np);
     B.res = (float*)take(12 * np);
     B.dwpart = (float*)take((size_t)kDwBlocks * 27 * 256 * 4);
-    B.dwsum = (float*)take(27 * 256 * 4);
+    take(27 * 256 * 4);  // (unused)
     B.bpart = (float*)take((size_t)kBiasBlocks * 16 * 4);
     B.lpart = (double*)take((size_t)kLossBlocks * 8);
     return B;
@@ -495,21 +567,6 @@ int net_forward(const cola_net* net, char* lbase, int ng, int nq, float green, f
     return check_launch();
 }
 
-// transposed weight-gradient sum [27][16][16] -> master layout [co][ci][27]
-__global__ void k_unpack_dw(const float* __restrict__ dwt, int co_n, int ci_n, float* __restrict__ out) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= co_n * ci_n * 27) return;
-    const int t = e % 27, ci = (e / 27) % ci_n, co = e / (27 * ci_n);
-    out[e] = dwt[(t * 16 + co) * 16 + ci];
-}
-
-__global__ void k_fix3_to_float(const unsigned long long* __restrict__ fix3, float* __restrict__ dF, long long n,
-                                float scale) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    dF[i] = (float)(long long)fix3[i] * scale;
-}
-
 static int layer_grads(const bf16* x, const bf16* dy, int ng, int co_n, int ci_n, float* gW, float* gb,
                        const LearnedBufs& B, cudaStream_t s) {
     static bool attr = false;
@@ -520,11 +577,10 @@ static int layer_grads(const bf16* x, const bf16* dy, int ng, int co_n, int ci_n
     }
     const long long n3 = (long long)ng * ng * ng;
     k_conv_dw<<<kDwBlocks, 288, kDwSmem, s>>>(x, dy, ng, B.dwpart);
-    k_sum_partials<<<(27 * 256 + 255) / 256, 256, 0, s>>>(B.dwpart, kDwBlocks, 27 * 256, B.dwsum);
-    k_unpack_dw<<<(co_n * ci_n * 27 + 255) / 256, 256, 0, s>>>(B.dwsum, co_n, ci_n, gW);
+    k_dw_finish<<<27 * 256 / 32, dim3(32, kSumRows), 0, s>>>(B.dwpart, kDwBlocks, co_n, ci_n, gW);
     k_bias_grad<<<kBiasBlocks, 256, 0, s>>>(dy, n3, co_n, B.bpart);
-    k_sum_partials<<<1, 32, 0, s>>>(B.bpart, kBiasBlocks, co_n, gb);
-    g_launches += 5;
+    k_db_finish<<<1, 512, 0, s>>>(B.bpart, kBiasBlocks, co_n, gb);
+    g_launches += 4;
     return check_launch();
 }
 
@@ -537,16 +593,15 @@ int net_backward(const cola_net* net, char* lbase, int ng, int nq, double box, f
     int rc;
     if ((rc = launch_gather(F, d, B.pred, nq, ng, box, s))) return rc;
     ProfScope ps(kKLearned, s);
-    k_residual<<<kLossBlocks, 256, 0, s>>>(B.pred, target, B.res, 3 * np, B.lpart);
-    k_sum_double<<<1, 32, 0, s>>>(B.lpart, kLossBlocks, 0.5 / (double)np, loss);
+    k_residual<<<kLossBlocks, kLossThreads, 0, s>>>(B.pred, target, B.res, 3 * np, B.lpart);
+    static_assert(kLossBlocks <= 512, "one block adds the partials");
+    k_sum_double<<<1, 512, 0, s>>>(B.lpart, kLossBlocks, 0.5 / (double)np, loss);
     if (cudaMemsetAsync(B.fix3, 0, 24 * (size_t)n3, s) != cudaSuccess) return COLA_ECUDA;
     if ((rc = launch_adjoint_deposit(d, B.res, B.fix3, nq, ng, box, s))) return rc;
-    // dL/dF_mesh = deposit / Np (2^-30 fixed point)
-    k_fix3_to_float<<<(unsigned)((3 * n3 + 255) / 256), 256, 0, s>>>(B.fix3, B.dF, 3 * n3,
-                                                                     (float)(1.0 / 1073741824.0 / (double)np));
-    // last layer: F += g out  ->  dL/dout = g dL/dF
-    k_pack_grad<<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(B.dF, ng, green, B.g1);
-    g_launches += 4;
+    // dL/dF_mesh = deposit / Np (2^-30 fixed point); last layer: F += g out  ->  dL/dout = g dL/dF
+    k_pack_grad<<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(B.fix3, ng, (float)(1.0 / 1073741824.0 / (double)np),
+                                                           green, B.g1);
+    g_launches += 3;
     if ((rc = layer_grads(B.h2, B.g1, ng, 3, 16, grad + kW3, grad + kB3, B, s))) return rc;
     k_conv<2, kEpiMask><<<conv_grid(ng), kConvWarps * 32, 0, s>>>(B.g1, wp + kPd3, nullptr, ng, B.g2, B.h2, nullptr,
                                                                   0, 0.f);
