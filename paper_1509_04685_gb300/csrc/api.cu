@@ -152,12 +152,10 @@ static int pm_mesh_forces(const cola_config* cfg, const cola_state* st, double g
         // the region marked clean
         unsigned long long* dep = reinterpret_cast<unsigned long long*>(wsp(ws, L.dep));
         if ((rc = clear_dep_if_dirty(ws, dep, (size_t)ng * ng * ng, s))) return rc;
-        if ((rc = mark_dep_dirty(ws, s))) return rc;
         if ((rc = launch_deposit_ex(st->d, nullptr, nullptr, nullptr, dep, nq, ng, cfg->box, nullptr, status_ptr(ws),
-                                    s, false)))
+                                    s, false, dep_state_ptr(ws))))
             return rc;
-        if ((rc = fft_z_r2c(dep, F, ng, scale, tw, s, P, n2, fr))) return rc;
-        if ((rc = mark_dep_clean(ws, s))) return rc;
+        if ((rc = fft_z_r2c(dep, F, ng, scale, tw, s, P, n2, fr, true, dep_state_ptr(ws)))) return rc;
     }
     const long long XB = 1ll << fr.xbs;
     // y lines of component 0 (outer x = xb XB + xi), then of all three components (outer 3 x + c)

@@ -472,7 +472,7 @@ constexpr size_t kHdrSnap = 128;          // 6 doubles: snapshot drift (dr, dD1,
 constexpr size_t kHdrProbe = 512;         // 64 ints written by cola_checks_probe
 constexpr int kProbeInts = 64;
 constexpr size_t kHdrDepState = 768;      // int: kDepClean while the fixed-point region holds zero counts
-constexpr int kDepClean = 0x5a5a5a5a;     // (a byte pattern, so cudaMemsetAsync can write it)
+constexpr int kDepClean = 0x5a5a5a5a;
 constexpr size_t kHdrFilter = 1024;       // radial filter basis table (<= 64 floats)
 constexpr size_t kHdrTable = 4096;        // kMaxSteps x kTableCols doubles
 constexpr size_t kHdrTwiddle = 262144;    // 3 slots of kMaxFft float2
@@ -592,9 +592,10 @@ int persistent_grid(size_t smem, int ntiles);
 int persistent_grid(size_t smem, int ntiles, int max_per_sm);
 // z passes: row r at base + r*rs (complex units), nrows rows
 // r2c: input row r = x n + y goes to output row frow(x, y, 0, fr) (fr = {n, 0, 1}: in place, same row)
-// dep: fixed-point counts to transform instead, cleared as they are read unless clear = false
+// dep: fixed-point counts to transform instead, cleared as they are read unless clear = false;
+// clean (optional, with clear): the region's state word, marked clean by the kernel itself
 int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const float2* tw, cudaStream_t s,
-              long long rs, long long nrows, FRow fr, bool clear = true);
+              long long rs, long long nrows, FRow fr, bool clear = true, int* clean = nullptr);
 int fft_z_c2r(float2* data, int n, const float2* tw, cudaStream_t s, float* out, long long opitch, float oscale,
               long long rs, long long nrows);
 // line passes: tile of outer index o starts at (o / o2n) s1 + (o % o2n) s2, element stride S
@@ -611,9 +612,11 @@ int fft_x_green(float2* F, int n, float gscale, float kf, const float2* tw, cuda
 int fft_y_inverse_force(float2* F, int n, const float2* tw, cudaStream_t s, bool psi, float kf);
 __host__ __device__ __forceinline__ FRow force_rows(int ng) { return FRow{ng, xblock_shift(ng), 3}; }
 
-// snap (optional): drift to an output time; rsd: also shift along z into redshift space (snap[3..5])
+// snap (optional): drift to an output time; rsd: also shift along z into redshift space (snap[3..5]);
+// dirty (optional): the region's state word, marked dirty by the kernel itself
 int launch_deposit_ex(const float* d, const float* v, const float* psi1, const float* psi2, unsigned long long* dep,
-                      int nq, int ng, double box, const double* snap, int* status, cudaStream_t s, bool rsd = false);
+                      int nq, int ng, double box, const double* snap, int* status, cudaStream_t s, bool rsd = false,
+                      int* dirty = nullptr);
 // F: interleaved force mesh, real view, component c of (ix, iy) at ((ix n + iy) 3 + c) 2P floats
 int launch_gather(const float2* F, const float* d, float* out, int nq, int ng, double box, cudaStream_t s);
 int launch_gather_kick_drift(const float2* F, cola_state st, const double* row, int nq, int ng, double box, int last,
@@ -641,9 +644,11 @@ int launch_slot_force(const float* slots, const int* pos, float* out, int nq, cu
 // r2c pass clears the counts as it reads them, so the region stays zero from
 // one such step to the next.  Everything else that writes the region (the
 // fused path's bins, the 2LPT scratch, the P(k) and density calls) marks it
-// dirty first; clear_dep_if_dirty zeroes it only when marked.
+// dirty first; clear_dep_if_dirty zeroes it only when marked.  In a step the
+// deposit and the z r2c pass write the state word themselves (two stream memsets
+// less, about 6 us of a small step).
 int mark_dep_dirty(void* ws, cudaStream_t s);
-int mark_dep_clean(void* ws, cudaStream_t s);
+inline int* dep_state_ptr(void* ws) { return reinterpret_cast<int*>(wsp(ws, kHdrDepState)); }
 int clear_dep_if_dirty(void* ws, unsigned long long* dep, size_t count, cudaStream_t s);
 // cola_checks_probe's kernel: area[index] = index if the bounds check index < n passes
 int launch_checks_probe(int* area, int index, int n, int* status, cudaStream_t s);

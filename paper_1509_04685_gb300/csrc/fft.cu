@@ -237,7 +237,8 @@ struct YZStore {
 template <bool FIX>
 __global__ void k_fft_z_r2c(unsigned long long* __restrict__ dep, float2* out, int n, long long rs, long long nrows,
                             int NR, float scale, FftPlan plan, const float2* __restrict__ tw, FastDiv m1div, FRow fr,
-                            bool clear) {
+                            bool clear, int* clean) {
+    if (clean && blockIdx.x == 0 && threadIdx.x == 0) *clean = kDepClean;
     extern __shared__ float2 sm[];
     __shared__ long long obase[64];  // output row offsets of this block's lines
     const int M = n / 2;
@@ -481,7 +482,7 @@ static int pass_threads(const FftPlan& plan, long lines) {
 }
 
 int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const float2* tw, cudaStream_t s,
-              long long rs, long long nrows, FRow fr, bool clear) {
+              long long rs, long long nrows, FRow fr, bool clear, int* clean) {
     FftPlan plan;
     if (!make_plan(n / 2, &plan)) return COLA_EUNSUPPORTED_SIZE;
     const int M = n / 2;
@@ -491,15 +492,15 @@ int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const fl
     const long long grid = (nrows + NR - 1) / NR;
     ProfScope ps(dep ? kKZr2cFix : kKZr2c, s);
     int rc = COLA_OK;
-    if (dep && launch_z_r2c_fix_static(dep, out, n, rs, nrows, scale, tw, fr, clear, s, &rc)) return rc;
+    if (dep && launch_z_r2c_fix_static(dep, out, n, rs, nrows, scale, tw, fr, clear, clean, s, &rc)) return rc;
     if (dep) {
         if (!set_smem((const void*)k_fft_z_r2c<true>, smem)) return COLA_ECUDA;
         k_fft_z_r2c<true><<<(unsigned)grid, T, smem, s>>>(dep, out, n, rs, nrows, NR, scale, plan, tw,
-                                                           make_fastdiv(M + 1), fr, clear);
+                                                           make_fastdiv(M + 1), fr, clear, clean);
     } else {
         if (!set_smem((const void*)k_fft_z_r2c<false>, smem)) return COLA_ECUDA;
         k_fft_z_r2c<false><<<(unsigned)grid, T, smem, s>>>(nullptr, out, n, rs, nrows, NR, 0.f, plan, tw,
-                                                            make_fastdiv(M + 1), fr, false);
+                                                            make_fastdiv(M + 1), fr, false, nullptr);
     }
     return check_launch();
 }
@@ -784,11 +785,8 @@ int fft_y_inverse_force(float2* F, int n, const float2* tw, cudaStream_t s, bool
     // lines of one component: outer x = xb XB + xi
     const LineGeom one{3 * XB * P, n, (int)XB, 3 * XB * n * P, 3 * P};
     int rc = COLA_OK;
-    if ((long long)n * nct <= 0x7fffffff &&
-        launch_y_psi_static(F + P, n, B, one, P, nct, n * nct, tw, kf, s, &rc)) {
-        if (rc) return rc;
-        return fft_lines(F, n, +1, tw, s, one, -1);
-    }
+    if (2ll * n * nct <= 0x7fffffff && launch_y_psi_static(F + P, n, B, one, P, -P, nct, n * nct, tw, kf, s, &rc))
+        return rc;  // F_x too
     const long long ne = (long long)n * n * (n / 2 + 1);
     k_expand_psi<<<(unsigned)((ne + 255) / 256), 256, 0, s>>>(F, n, (int)P, fr.xbs, kf);
     if ((rc = check_launch())) return rc;

@@ -90,7 +90,7 @@ bool launch_x_green_static(float2* F, int n, int B, int nct, int ntiles, const f
 
 // default column width of the specialised line passes of each size
 static const int kStaticTiles[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {288, 16}, {320, 16}, {384, 16}, {480, 16}, {512, 16}, {768, 16}, {1024, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
-static const int kStaticSpecs[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {256, 8}, {288, 16}, {320, 16}, {384, 16}, {384, 8}, {480, 16}, {480, 8}, {512, 16}, {512, 8}, {1024, 8}, {768, 16}, {768, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
+static const int kStaticSpecs[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {256, 8}, {288, 16}, {320, 16}, {384, 16}, {384, 8}, {480, 16}, {480, 8}, {512, 16}, {512, 8}, {1024, 8}, {768, 16}, {1152, 8}, {1536, 8}, {2304, 4}};
 
 // default column width of the specialised fused x/Green pass of each size
 static const int kGreenTiles[][2] = {{768, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
@@ -148,13 +148,13 @@ bool static_tile_ok(int n, int B) {
 
 template <int N, int W, int MB>
 static int run_z_r2c_fix_w(unsigned long long* dep, float2* out, long long rs, long long nrows, float scale,
-                           const float2* tw, FRow fr, bool clear, cudaStream_t s) {
+                           const float2* tw, FRow fr, bool clear, int* clean, cudaStream_t s) {
     constexpr size_t smem = z_warp_smem<N, W>();
     static_assert((smem + 1024) * MB <= 227 * 1024, "MB blocks must fit");
     if (!set_smem((const void*)k_fft_z_r2c_fix_w<N, W, MB>, smem)) return COLA_ECUDA;
     const long long units = (nrows + W - 1) / W;
     k_fft_z_r2c_fix_w<N, W, MB><<<persistent_grid(smem, (int)(units < 0x7fffffff ? units : 0x7fffffff), MB),
-                                  32 * W, smem, s>>>(dep, out, rs, nrows, scale, tw, fr, clear);
+                                  32 * W, smem, s>>>(dep, out, rs, nrows, scale, tw, fr, clear, clean);
     return check_launch();
 }
 
@@ -172,22 +172,22 @@ bool launch_z_c2r_static(float2* data, int n, long long rs, long long nrows, con
 }
 
 bool launch_z_r2c_fix_static(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
-                             float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc) {
+                             float scale, const float2* tw, FRow fr, bool clear, int* clean, cudaStream_t s, int* rc) {
 #define COLA_CASE(NN, WW, MB)                                                               \
     if (n == NN && nrows == (long long)NN * NN) {                                          \
-        *rc = run_z_r2c_fix_w<NN, WW, MB>(dep, out, rs, nrows, scale, tw, fr, clear, s);    \
+        *rc = run_z_r2c_fix_w<NN, WW, MB>(dep, out, rs, nrows, scale, tw, fr, clear, clean, s);    \
         return true;                                                                        \
     }
     COLA_ZWARP_SPECS(COLA_CASE)
 #undef COLA_CASE
 #define COLA_CASE(NN, RR, TT, MB)                                                   \
     if (n == NN) {                                                                  \
-        *rc = run_z_r2c_fix<NN, RR, TT, MB>(dep, out, rs, nrows, scale, tw, fr, clear, s); \
+        *rc = run_z_r2c_fix<NN, RR, TT, MB>(dep, out, rs, nrows, scale, tw, fr, clear, clean, s); \
         return true;                                                                \
     }
     COLA_ZR2C_SPECS(COLA_CASE)
 #undef COLA_CASE
-    return launch_z_r2c_fix_static_small(dep, out, n, rs, nrows, scale, tw, fr, clear, s, rc);
+    return launch_z_r2c_fix_static_small(dep, out, n, rs, nrows, scale, tw, fr, clear, clean, s, rc);
 }
 
 
@@ -282,23 +282,24 @@ bool launch_z_c2r_gather_static(float2* data, int n, long long rs, const float2*
     return false;
 }
 
-bool launch_y_psi_static(float2* data, int n, int B, LineGeom lg, long long comp2, int nct, int ntiles,
+bool launch_y_psi_static(float2* data, int n, int B, LineGeom lg, long long comp2, long long comp0, int nct, int ntiles,
                          const float2* tw, float kf, cudaStream_t s, int* rc) {
 #define COLA_CASE(NN, BB, TT)                                                     \
     if (n == NN && B == BB) {                                                     \
-        *rc = run_y_psi2<NN, BB, TT>(data, lg, comp2, nct, ntiles, tw, kf, s);   \
+        *rc = run_y_psi2<NN, BB, TT>(data, lg, comp2, nct, ntiles, tw, kf, s);    \
+        if (!*rc) launch_strided_static(data + comp0, n, B, +1, lg, nct, ntiles, tw, s, rc); \
         return true;                                                              \
     }
     COLA_YPSI2_SPECS(COLA_CASE)
 #undef COLA_CASE
 #define COLA_CASE(NN, BB, TT)                                                   \
     if (n == NN && B == BB) {                                                   \
-        *rc = run_y_psi<NN, BB, TT>(data, lg, comp2, nct, ntiles, tw, kf, s); \
+        *rc = run_y_psi<NN, BB, TT>(data, lg, comp2, comp0, nct, ntiles, tw, kf, s); \
         return true;                                                            \
     }
     COLA_STRIDED_SPECS(COLA_CASE)
 #undef COLA_CASE
-    return launch_y_psi_static_small(data, n, B, lg, comp2, nct, ntiles, tw, kf, s, rc);
+    return launch_y_psi_static_small(data, n, B, lg, comp2, comp0, nct, ntiles, tw, kf, s, rc);
 }
 
 }  // namespace cola

@@ -62,11 +62,11 @@ bool launch_x_green_static_small(float2* F, int n, int B, int nct, int ntiles, c
 int launch_static_green_tile_small(int) { return 0; }
 
 
-bool launch_y_psi_static_small(float2* data, int n, int B, LineGeom lg, long long comp2, int nct, int ntiles,
+bool launch_y_psi_static_small(float2* data, int n, int B, LineGeom lg, long long comp2, long long comp0, int nct, int ntiles,
                          const float2* tw, float kf, cudaStream_t s, int* rc) {
 #define COLA_CASE(NN, BB, TT)                                                   \
     if (n == NN && B == BB) {                                                   \
-        *rc = run_y_psi<NN, BB, TT>(data, lg, comp2, nct, ntiles, tw, kf, s); \
+        *rc = run_y_psi<NN, BB, TT>(data, lg, comp2, comp0, nct, ntiles, tw, kf, s); \
         return true;                                                            \
     }
     COLA_STRIDED_SPECS(COLA_CASE)
@@ -101,10 +101,10 @@ bool launch_z_c2r_static_small(float2* data, int n, long long rs, long long nrow
 }
 
 bool launch_z_r2c_fix_static_small(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
-                                   float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc) {
+                                   float scale, const float2* tw, FRow fr, bool clear, int* clean, cudaStream_t s, int* rc) {
 #define COLA_CASE(NN, RR, TT, M1, M2)                                                      \
     if (n == NN) {                                                                         \
-        *rc = run_z_r2c_fix<NN, RR, TT, M2>(dep, out, rs, nrows, scale, tw, fr, clear, s); \
+        *rc = run_z_r2c_fix<NN, RR, TT, M2>(dep, out, rs, nrows, scale, tw, fr, clear, clean, s); \
         return true;                                                                       \
     }
     COLA_Z_SPECS(COLA_CASE)

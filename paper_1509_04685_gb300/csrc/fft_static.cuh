@@ -624,9 +624,13 @@ struct SColIkz {
 // tile of Psi gives F_y = IFFT_y(i k_y Psi) (k_y varies along the y line) into
 // component 1 and F_z = i k_z IFFT_y(Psi) (k_z is the column's, constant along
 // the line) into component 2.  lg addresses component 1; component 2 follows
-// at + comp2.
+// at + comp2.  With comp0 the same launch also transforms component 0 (F_x) at
+// + comp0, its tiles after the others: one launch less per step (a step of 32^3
+// particles on 96^3 is a dozen launches of 3 to 9 us and the gaps between them).
+// The two-lines-per-thread form of the large meshes keeps the passes apart:
+// together they took 2.03 ms against 1.93 at 768 and 7.31 against 6.76 at 1152.
 template <int N, int B, int T>
-__global__ void __launch_bounds__(T, 1) k_fft_y_psi_s(float2* data, LineGeom lg, long long comp2, int nct, int ntiles,
+__global__ void __launch_bounds__(T, 1) k_fft_y_psi_s(float2* data, LineGeom lg, long long comp2, long long comp0, int nct, int ntiles,
                                                        const float2* __restrict__ tw, float kf) {
     using Geo = ColTile<B>;
     constexpr int TSZ = spad(N) * B;
@@ -635,25 +639,32 @@ __global__ void __launch_bounds__(T, 1) k_fft_y_psi_s(float2* data, LineGeom lg,
     float2* A = sm + TSZ;
     float2* tws = A + TSZ;
     for (int q = threadIdx.x; q < N; q += T) tws[q] = __ldg(tw + q);
+    const int ntot = comp0 ? 2 * ntiles : ntiles;
     const SCol rows{nullptr, lg.S};
     auto tile_base = [&](int t) {
+        const long long comp = t < ntiles ? 0 : comp0;
+        if (t >= ntiles) t -= ntiles;
         const int o = t / nct;
         const int ct = t - o * nct;
         const int o1 = o / lg.o2n, o2 = o - o1 * lg.o2n;
-        return data + o1 * lg.s1 + o2 * lg.s2 + ct * B;
+        return data + comp + o1 * lg.s1 + o2 * lg.s2 + ct * B;
     };
     int t = blockIdx.x;
-    if (t < ntiles) stile_prefetch<N, B, T>(stg, tile_base(t), rows);
-    for (; t < ntiles; t += gridDim.x) {
+    if (t < ntot) stile_prefetch<N, B, T>(stg, tile_base(t), rows);
+    for (; t < ntot; t += gridDim.x) {
         cp_async_wait_all();
         __syncthreads();
         float2* base = tile_base(t);
-        const int col0 = (t - (t / nct) * nct) * B;
-        sip_run<N, T, Geo, +1, false, false>(IkxLoad<N, Geo>{stg, kf}, SCol{base, lg.S}, A, tws, NoHook{});
         const int tn = t + gridDim.x;
         auto next = [&]() {
-            if (tn < ntiles) stile_prefetch<N, B, T>(stg, tile_base(tn), rows);
+            if (tn < ntot) stile_prefetch<N, B, T>(stg, tile_base(tn), rows);
         };
+        if (t >= ntiles) {  // F_x
+            sip_run<N, T, Geo, +1, false, false>(SSmem<Geo>{stg}, SCol{base, lg.S}, A, tws, next);
+            continue;
+        }
+        const int col0 = (t - (t / nct) * nct) * B;
+        sip_run<N, T, Geo, +1, false, false>(IkxLoad<N, Geo>{stg, kf}, SCol{base, lg.S}, A, tws, NoHook{});
         sip_run<N, T, Geo, +1, false, false>(SSmem<Geo>{stg}, SColIkz{base + comp2, lg.S, kf, col0, N / 2}, A, tws,
                                              next);
     }
@@ -868,11 +879,12 @@ inline int run_y_psi2(float2* data, LineGeom lg, long long comp2, int nct, int n
 }
 
 template <int N, int B, int T>
-inline int run_y_psi(float2* data, LineGeom lg, long long comp2, int nct, int ntiles, const float2* tw, float kf,
-                     cudaStream_t s) {
+inline int run_y_psi(float2* data, LineGeom lg, long long comp2, long long comp0, int nct, int ntiles,
+                     const float2* tw, float kf, cudaStream_t s) {
     const size_t smem = ((size_t)2 * spad(N) * B + N) * 8;
     if (!set_smem((const void*)k_fft_y_psi_s<N, B, T>, smem)) return COLA_ECUDA;
-    k_fft_y_psi_s<N, B, T><<<persistent_grid(smem, ntiles), T, smem, s>>>(data, lg, comp2, nct, ntiles, tw, kf);
+    k_fft_y_psi_s<N, B, T><<<persistent_grid(smem, comp0 ? 2 * ntiles : ntiles), T, smem, s>>>(data, lg, comp2, comp0, nct,
+                                                                                         ntiles, tw, kf);
     return check_launch();
 }
 
@@ -1163,7 +1175,9 @@ constexpr size_t z_warp_smem() {
 template <int N, int W, int MB>
 __global__ void __launch_bounds__(32 * W, MB) k_fft_z_r2c_fix_w(unsigned long long* __restrict__ dep, float2* out,
                                                                long long rs, long long nrows, float scale,
-                                                               const float2* __restrict__ tw, FRow fr, bool clear) {
+                                                               const float2* __restrict__ tw, FRow fr, bool clear,
+                                                               int* clean) {
+    if (clean && blockIdx.x == 0 && threadIdx.x == 0) *clean = kDepClean;
     constexpr int M = N / 2;
     using Geo = WarpRow<M>;
     extern __shared__ float2 sm[];
@@ -1249,7 +1263,9 @@ __global__ void __launch_bounds__(T, MB) k_fft_z_c2r_s(float2* data, long long r
 template <int N, int NR, int T, int MB>
 __global__ void __launch_bounds__(T, MB) k_fft_z_r2c_fix_s(unsigned long long* __restrict__ dep, float2* out,
                                                             long long rs, long long nrows, int ntiles, float scale,
-                                                            const float2* __restrict__ tw, FRow fr, bool clear) {
+                                                            const float2* __restrict__ tw, FRow fr, bool clear,
+                                                               int* clean) {
+    if (clean && blockIdx.x == 0 && threadIdx.x == 0) *clean = kDepClean;
     constexpr int M = N / 2;
     using Geo = RowTile<M, NR>;
     constexpr int HN = N / 2;  // 16-byte chunks per count row
@@ -1325,14 +1341,14 @@ inline int run_z_c2r(float2* data, long long rs, long long nrows, const float2* 
 
 template <int N, int NR, int T, int MB>
 inline int run_z_r2c_fix(unsigned long long* dep, float2* out, long long rs, long long nrows, float scale,
-                         const float2* tw, FRow fr, bool clear, cudaStream_t s) {
+                         const float2* tw, FRow fr, bool clear, int* clean, cudaStream_t s) {
     constexpr size_t smem = z_r2c_smem<N, NR, T>();
     static_assert((smem + 64 * NR + 1024) * MB <= 227 * 1024, "MB blocks must fit in shared memory");
     const long long nt = (nrows + NR - 1) / NR;
     if (nt > 0x7fffffff) return COLA_EUNSUPPORTED_SIZE;
     if (!set_smem((const void*)k_fft_z_r2c_fix_s<N, NR, T, MB>, smem)) return COLA_ECUDA;
     k_fft_z_r2c_fix_s<N, NR, T, MB><<<persistent_grid(smem, (int)nt, MB), T, smem, s>>>(dep, out, rs, nrows, (int)nt,
-                                                                                     scale, tw, fr, clear);
+                                                                                     scale, tw, fr, clear, clean);
     return check_launch();
 }
 
@@ -1347,11 +1363,11 @@ bool launch_x_green_static(float2* F, int n, int B, int nct, int ntiles, const f
 bool launch_z_c2r_static(float2* data, int n, long long rs, long long nrows, const float2* tw, cudaStream_t s,
                          int* rc);
 bool launch_z_r2c_fix_static(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
-                             float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc);
+                             float scale, const float2* tw, FRow fr, bool clear, int* clean, cudaStream_t s, int* rc);
 bool launch_z_c2r_static_small(float2* data, int n, long long rs, long long nrows, const float2* tw, cudaStream_t s,
                                int* rc);
 bool launch_z_r2c_fix_static_small(unsigned long long* dep, float2* out, int n, long long rs, long long nrows,
-                                   float scale, const float2* tw, FRow fr, bool clear, cudaStream_t s, int* rc);
+                                   float scale, const float2* tw, FRow fr, bool clear, int* clean, cudaStream_t s, int* rc);
 // default column width of the specialised line passes for n (0: none)
 int static_tile(int n);
 // whether (n, B) has specialised line passes
@@ -1362,10 +1378,10 @@ int static_green_tile(int n);
 int launch_static_green_tile_small(int n);
 // inverse y pass of the Psi component (k_fft_y_psi_s) for (n, B); false when
 // there is no specialisation, without launching
-bool launch_y_psi_static(float2* data, int n, int B, LineGeom lg, long long comp2, int nct, int ntiles,
-                         const float2* tw, float kf, cudaStream_t s, int* rc);
-bool launch_y_psi_static_small(float2* data, int n, int B, LineGeom lg, long long comp2, int nct, int ntiles,
-                               const float2* tw, float kf, cudaStream_t s, int* rc);
+bool launch_y_psi_static(float2* data, int n, int B, LineGeom lg, long long comp2, long long comp0, int nct,
+                         int ntiles, const float2* tw, float kf, cudaStream_t s, int* rc);
+bool launch_y_psi_static_small(float2* data, int n, int B, LineGeom lg, long long comp2, long long comp0,
+                               int nct, int ntiles, const float2* tw, float kf, cudaStream_t s, int* rc);
 // the mesh sizes below 512 (batched ensembles, tests), in fft_spec_small.cu
 bool launch_strided_static_small(float2* data, int n, int B, int sign, LineGeom lg, int nct, int ntiles,
                                  const float2* tw, cudaStream_t s, int* rc);

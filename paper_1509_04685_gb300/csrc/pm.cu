@@ -112,7 +112,9 @@ __device__ __forceinline__ long long site_index(const int idx[3], int nq) {
 template <bool SNAP, bool RSD = false>
 __global__ void k_deposit(const float* __restrict__ d, const float* __restrict__ v, const float* __restrict__ psi1,
                           const float* __restrict__ psi2, unsigned long long* __restrict__ dep, int nq, int ng,
-                          float inv_cell, long long np, const double* __restrict__ snap, int* status, Trav tv) {
+                          float inv_cell, long long np, const double* __restrict__ snap, int* status, Trav tv,
+                          int* dirty) {
+    if (dirty && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x) == 0) *dirty = 0;
     int idx[3];
     if (!trav_site(tv, idx)) return;
     const long long p = site_index(idx, nq);
@@ -149,7 +151,7 @@ __global__ void k_deposit(const float* __restrict__ d, const float* __restrict__
 }
 
 int launch_deposit_ex(const float* d, const float* v, const float* psi1, const float* psi2, unsigned long long* dep,
-                      int nq, int ng, double box, const double* snap, int* status, cudaStream_t s, bool rsd) {
+                      int nq, int ng, double box, const double* snap, int* status, cudaStream_t s, bool rsd, int* dirty) {
     const long long np = (long long)nq * nq * nq;
     const Trav tv = make_trav(nq);
     const dim3 grid = trav_grid(tv);
@@ -157,11 +159,11 @@ int launch_deposit_ex(const float* d, const float* v, const float* psi1, const f
     const float inv_cell = (float)((double)ng / box);
     ProfScope ps(kKDeposit, s);
     if (snap && rsd)
-        k_deposit<true, true><<<grid, T, 0, s>>>(d, v, psi1, psi2, dep, nq, ng, inv_cell, np, snap, status, tv);
+        k_deposit<true, true><<<grid, T, 0, s>>>(d, v, psi1, psi2, dep, nq, ng, inv_cell, np, snap, status, tv, dirty);
     else if (snap)
-        k_deposit<true><<<grid, T, 0, s>>>(d, v, psi1, psi2, dep, nq, ng, inv_cell, np, snap, status, tv);
+        k_deposit<true><<<grid, T, 0, s>>>(d, v, psi1, psi2, dep, nq, ng, inv_cell, np, snap, status, tv, dirty);
     else
-        k_deposit<false><<<grid, T, 0, s>>>(d, v, psi1, psi2, dep, nq, ng, inv_cell, np, nullptr, status, tv);
+        k_deposit<false><<<grid, T, 0, s>>>(d, v, psi1, psi2, dep, nq, ng, inv_cell, np, nullptr, status, tv, dirty);
     return check_launch();
 }
 
@@ -493,11 +495,6 @@ int launch_slot_force(const float* slots, const int* pos, float* out, int nq, cu
 
 int mark_dep_dirty(void* ws, cudaStream_t s) {
     return cudaMemsetAsync(wsp(ws, kHdrDepState), 0, sizeof(int), s) == cudaSuccess ? COLA_OK : COLA_ECUDA;
-}
-
-int mark_dep_clean(void* ws, cudaStream_t s) {
-    return cudaMemsetAsync(wsp(ws, kHdrDepState), kDepClean & 0xff, sizeof(int), s) == cudaSuccess ? COLA_OK
-                                                                                                   : COLA_ECUDA;
 }
 
 // zero count[0 .. n) (n even) unless the state word says it is already zero
