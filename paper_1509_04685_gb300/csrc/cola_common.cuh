@@ -197,6 +197,10 @@ template <>
 struct SmallDft<12> {
     __device__ __forceinline__ static void run(float2* v, int sign) { pfa_dft<4, 3>(v, sign); }
 };
+template <>
+struct SmallDft<24> {
+    __device__ __forceinline__ static void run(float2* v, int sign) { pfa_dft<8, 3>(v, sign); }
+};
 
 // ---------------------------------------------------------------------------
 // FFT plan: n = product of radices (applied in order), n <= kMaxFft

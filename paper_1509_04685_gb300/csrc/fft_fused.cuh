@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(96 * TX * G, MB)
 // barriers (id g + 1) separate the phases.
 template <int N, int NR, int G>
 constexpr int z_r2c_dep_w_tw() {  // float2 entries before the counts (16-byte aligned)
-    return (ordered_tw_size(N / 2) + N / 2 + 1 + 1) & ~1;
+    return (warp_tw_size<N / 2>() + N / 2 + 1 + 1) & ~1;
 }
 template <int N, int NR, int G>
 constexpr size_t z_r2c_dep_w_smem() {
@@ -547,9 +547,9 @@ __global__ void __launch_bounds__(32 * NR * G, MB)
     extern __shared__ float2 sm[];
     __shared__ int beg[G][NB], pre[G][NB + 1], bxy[G][NB];
     float2* tws = sm;                        // pass-ordered twiddles of the M-point transform
-    float2* twh = tws + ordered_tw_size(M);  // W_N^k, k <= M, for the r2c post-processing
+    float2* twh = tws + warp_tw_size<M>();  // W_N^k, k <= M, for the r2c post-processing
     unsigned long long* cnt_all = reinterpret_cast<unsigned long long*>(sm + z_r2c_dep_w_tw<N, NR, G>());
-    ordered_twiddles<M, GT * G, 2>(tws, tw);
+    ordered_twiddles<M, GT * G, 2, WarpPlan<M>>(tws, tw);
     for (int q = threadIdx.x; q <= M; q += GT * G) twh[q] = __ldg(tw + q);
     __syncthreads();
     const int g = threadIdx.x / GT, gl = threadIdx.x - g * GT, l = gl >> 5, lane = gl & 31;
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(32 * NR * G, MB)
             float* o = delta_out + ((long long)x * N + y0 + l) * N;
             for (int e = lane; e < N; e += 32) o[e] = (float)fix_count(myc[e], split) * scale - 1.0f;
         }
-        sip_run<M, 32, Geo, -1, true, true>(FixCounts<N>{myc, scale, split}, SSmem<Geo>{Z}, Z, tws, NoHook());
+        sip_run<M, 32, Geo, -1, true, true, WarpPlan<M>>(FixCounts<N>{myc, scale, split}, SSmem<Geo>{Z}, Z, tws, NoHook());
         // X[k] = E[k] + W^k O[k], E = (Z[k] + conj Z[M-k]) / 2, O = (Z[k] - conj Z[M-k]) / (2i)
         float2* orow = out + frow(x, y0 + l, 0, fr) * rs;
         for (int k = lane; k <= M; k += 32) {

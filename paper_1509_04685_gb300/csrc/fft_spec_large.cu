@@ -8,22 +8,12 @@ namespace cola {
 // (n, B, threads) of every specialisation: B adjacent columns per tile, two
 // tile buffers of spad(n) B complex in shared memory
 #define COLA_STRIDED_SPECS(X) \
-    X(512, 16, 512) \
-    X(1024, 8, 512) \
-    X(768, 16, 1024) \
-    X(768, 8, 512) \
-    X(1152, 8, 1024) \
-    X(1536, 8, 1024) \
-    X(2304, 4, 1024)
+    X(768, 8, 512)
 
 #define COLA_XGREEN_SPECS(X) \
-    X(768, 16, 768, 2)       \
     X(768, 8, 1024, 3)       \
-    X(1152, 8, 768, 2)       \
     X(1152, 4, 768, 3)       \
-    X(1536, 8, 768, 2)       \
     X(1536, 4, 1024, 3)      \
-    X(2304, 4, 768, 2)       \
     X(2304, 2, 768, 3)
 
 // (n, B, threads) of the strided passes with two lines per thread; they take precedence
@@ -93,7 +83,7 @@ static const int kStaticTiles[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16},
 static const int kStaticSpecs[][2] = {{96, 16}, {128, 16}, {160, 16}, {192, 16}, {256, 16}, {256, 8}, {288, 16}, {320, 16}, {384, 16}, {384, 8}, {480, 16}, {480, 8}, {512, 16}, {512, 8}, {1024, 8}, {768, 16}, {1152, 8}, {1536, 8}, {2304, 4}};
 
 // default column width of the specialised fused x/Green pass of each size
-static const int kGreenTiles[][2] = {{768, 8}, {1152, 8}, {1536, 8}, {2304, 4}};
+static const int kGreenTiles[][2] = {{1152, 8}, {1536, 8}, {2304, 4}};
 
 int static_green_tile(int n) {
     for (const auto& e : kGreenTiles)

@@ -69,17 +69,20 @@ __host__ __device__ constexpr int tw_offset(const StaticPlan& p, int s) {
     }
     return off;
 }
-__host__ __device__ constexpr bool same_plan(const StaticPlan& a, const StaticPlan& b) {
-    if (a.nr != b.nr) return false;
-    for (int i = 0; i < a.nr; ++i)
-        if (a.r[i] != b.r[i]) return false;
-    return true;
-}
+// Radix order of a transform: the default plan of N, or three given radices.
+// Any order computes the same transform (the Stockham passes accumulate LS);
+// orders are chosen so that the in-place passes hold few values per thread.
+template <int N, int R0 = 0, int R1 = 0, int R2 = 0>
+struct PlanOf {
+    static constexpr StaticPlan P = R0 ? StaticPlan{true, 3, {R0, R1, R2}} : static_plan(N);
+    static_assert(R0 == 0 || R0 * R1 * R2 == N, "radices must multiply to N");
+};
+
 // Fill the pass-ordered table of an N-point plan in shared memory from the
 // table tw of N TWM entries exp(-2 pi i q / (N TWM)) (the same values).
-template <int N, int T, int TWM>
+template <int N, int T, int TWM, class PL = PlanOf<N>>
 __device__ __forceinline__ void ordered_twiddles(float2* out, const float2* __restrict__ tw) {
-    constexpr StaticPlan P = static_plan(N);
+    constexpr StaticPlan P = PL::P;
     int ls = P.r[0], off = 0;
     for (int s = 1; s < P.nr; ++s) {
         const int R = P.r[s], tws = N / (ls * R) * TWM;
@@ -202,15 +205,6 @@ __device__ __forceinline__ float2* srun_smem(const In& in, float2* a, float2* b,
     return res;
 }
 
-// Radix order of a transform: the default plan of N, or three given radices.
-// Any order computes the same transform (the Stockham passes accumulate LS);
-// orders are chosen so that the in-place passes hold few values per thread.
-template <int N, int R0 = 0, int R1 = 0, int R2 = 0>
-struct PlanOf {
-    static constexpr StaticPlan P = R0 ? StaticPlan{true, 3, {R0, R1, R2}} : static_plan(N);
-    static_assert(R0 == 0 || R0 * R1 * R2 == N, "radices must multiply to N");
-};
-
 // In-place pass: every butterfly of the thread is loaded into registers, the
 // block synchronises, then the butterflies are computed and stored over the
 // same buffer.  A tile then needs one working buffer instead of a ping-pong
@@ -270,7 +264,6 @@ __device__ __forceinline__ void sip_tail(float2* a, const Out& out, const float2
     constexpr StaticPlan P = PL::P;
     constexpr int R = P.r[S];
     constexpr int LS = plan_ls(P, S);
-    static_assert(!Geo::TWO || same_plan(P, static_plan(N)), "pass-ordered twiddles are laid out for the default plan");
     const float2* twp = Geo::TWO ? tw + tw_offset(P, S) : tw;
     if constexpr (S == P.nr - 1) {
         if constexpr (LAST_IP)
@@ -399,19 +392,6 @@ struct GreenPlans {
     using I1 = PlanOf<N>;
     using I2 = PlanOf<N>;
 };
-template <>
-struct GreenPlans<1536> {
-    using F = PlanOf<1536, 12, 8, 16>;
-    using I1 = PlanOf<1536, 12, 8, 16>;
-    using I2 = PlanOf<1536, 16, 8, 12>;
-};
-template <>
-struct GreenPlans<768> {
-    using F = PlanOf<768, 12, 4, 16>;
-    using I1 = PlanOf<768, 12, 4, 16>;
-    using I2 = PlanOf<768, 16, 4, 12>;
-};
-
 // strided complex pass (y: S = row stride, outer = x; or x on a plain mesh):
 // persistent blocks; the first pass reads the staged tile into the working
 // buffer, after which the next tile is staged with cp.async while the other
@@ -444,6 +424,15 @@ __global__ void __launch_bounds__(T, 1) k_fft_strided_s(float2* data, LineGeom l
         };
         sip_run<N, T, Geo, SIGN, false, false>(SSmem<Geo>{stg}, SCol{tile_base(t), lg.S}, A, tws, next);
     }
+}
+
+// radial transfer T(|k|), piecewise linear on nodes b * fstep
+__device__ __forceinline__ float radial_filter(float k2, const float* __restrict__ filt, int nfilt, float fstep) {
+    const float u = sqrtf(k2) / fstep;
+    int b = (int)u;
+    if (b > nfilt - 2) b = nfilt - 2;
+    const float f = fminf(u - (float)b, 1.f);
+    return (1.f - f) * filt[b] + f * filt[b + 1];
 }
 
 // x pass fused with the Poisson solve and the ik gradient on the interleaved,
@@ -500,14 +489,7 @@ __global__ void __launch_bounds__(T, 1) k_fft_x_green_s(float2* F, int nct, int 
             const float kx = kf * (float)(i < half ? i : i - N);
             const float k2 = kx * kx + kyz2;
             float gk = k2 > 0.f ? gscale / k2 : 0.f;
-            if (filt) {
-                // radial transfer T(|k|), piecewise linear on nodes b * fstep
-                const float u = sqrtf(k2) / fstep;
-                int b = (int)u;
-                if (b > nfilt - 2) b = nfilt - 2;
-                const float f = fminf(u - (float)b, 1.f);
-                gk *= (1.f - f) * filt[b] + f * filt[b + 1];
-            }
+            if (filt) gk *= radial_filter(k2, filt, nfilt, fstep);
             float2& x = elem(A, q);
             x = cscale(x, gk);
         }
@@ -576,14 +558,7 @@ __global__ void __launch_bounds__(T, 1) k_fft_x_green3_s(float2* F, int nct, int
             const float kx = kf * (float)(i < half ? i : i - N);
             const float k2 = kx * kx + kyz2;
             float gk = k2 > 0.f ? gscale / k2 : 0.f;
-            if (filt) {
-                // radial transfer T(|k|), piecewise linear on nodes b * fstep
-                const float u = sqrtf(k2) / fstep;
-                int b = (int)u;
-                if (b > nfilt - 2) b = nfilt - 2;
-                const float f = fminf(u - (float)b, 1.f);
-                gk *= (1.f - f) * filt[b] + f * filt[b + 1];
-            }
+            if (filt) gk *= radial_filter(k2, filt, nfilt, fstep);
             phi[q] = cscale(elem(X, q), gk);
         }
         __syncthreads();
@@ -956,30 +931,62 @@ struct SX2IO {
     }
 };
 
-// k_fft_x_green_s with two lines per thread in its transforms
+// Radix orders of k_fft_x_green2_s: the forward transform (first, second, R) and
+// the inverses (R, second, last).  R is the forward's last and the inverses' first
+// radix: the thread that ends up with the spectrum values k + r N/R of a butterfly
+// is the one that needs them, so the Green's function and the first inverse pass
+// of both transforms happen in its registers.
+template <int N>
+struct GreenRadices;
+template <>
+struct GreenRadices<512> {
+    static constexpr int F0 = 2, F1 = 16, R = 16, I1 = 16, I2 = 2;
+};
+template <>
+struct GreenRadices<768> {
+    static constexpr int F0 = 12, F1 = 4, R = 16, I1 = 4, I2 = 12;
+};
+template <>
+struct GreenRadices<1024> {
+    static constexpr int F0 = 4, F1 = 16, R = 16, I1 = 16, I2 = 4;
+};
+template <>
+struct GreenRadices<1152> {
+    static constexpr int F0 = 8, F1 = 12, R = 12, I1 = 12, I2 = 8;
+};
+template <>
+struct GreenRadices<1536> {
+    static constexpr int F0 = 12, F1 = 8, R = 16, I1 = 8, I2 = 12;
+};
+template <>
+struct GreenRadices<2304> {
+    static constexpr int F0 = 16, F1 = 12, R = 12, I1 = 12, I2 = 16;
+};
+
+// k_fft_x_green_s with two lines per thread and the middle of the pass in
+// registers: of the passes through shared memory of the three transforms and the
+// Green's function in between (ten reads and nine writes per value) five and five
+// are gone, and half of the block's barriers: 15.8 ms against 17.3 at 1536, 8.06
+// against 8.67 at 1152, 1.77 against 1.90 at 768 (the three-buffer form of eight
+// columns).  The latency of the accesses and barriers that remain still bounds it,
+// at twelve warps per SM.
 template <int N, int B, int T>
 __global__ void __launch_bounds__(T, 1) k_fft_x_green2_s(float2* F, int nct, int ntiles, const float2* __restrict__ tw,
                                                        float gscale, float kf, const float* __restrict__ filt,
                                                        int nfilt, float fstep) {
     using G = XGeom<N>;
+    using Q = GreenRadices<N>;
+    constexpr int R = Q::R, LS = N / R, NP = B / 2;
+    static_assert(Q::F0 * Q::F1 * R == N && Q::I1 * Q::I2 * R == N, "radices must multiply to N");
+    static_assert(LS * NP == T, "one middle butterfly per thread");
     constexpr int TSZ = spad(N) * B;
-    constexpr int TB = T / B;    // line-element stride between a thread's spectrum values
-    constexpr int EPT = N / TB;  // spectrum values per thread
-    static_assert(T % B == 0 && N % TB == 0, "tile must split evenly over the block");
     constexpr int half = N / 2;
     extern __shared__ float2 sm[];
     float2* stg = sm;
     float2* A = sm + TSZ;
     float2* tws = A + TSZ;
     for (int q = threadIdx.x; q < N; q += T) tws[q] = __ldg(tw + q);
-    const int c = threadIdx.x % B;   // this thread's column in the Green phase
-    const int i0 = threadIdx.x / B;  // and its first line element: i = i0 + q TB
-    auto elem = [&](float2* base, int q) -> float2& {
-        if constexpr (TB % 16 == 0)
-            return base[c + spad(i0) * B + q * spad(TB) * B];
-        else
-            return base[c + spad(i0 + q * TB) * B];
-    };
+    const int l2 = threadIdx.x % NP, j = threadIdx.x / NP;  // this thread's line pair and middle butterfly
     auto tile_off = [&](int t) {
         const int iy = t / nct;
         return (long long)iy * G::RS + (long long)(t - iy * nct) * B;
@@ -993,34 +1000,63 @@ __global__ void __launch_bounds__(T, 1) k_fft_x_green2_s(float2* F, int nct, int
         const long long off = (long long)iy * G::RS + col0;
         cp_async_wait_all();
         __syncthreads();
-        sip2_run<N, T, B, -1, false, true, typename GreenPlans<N>::F>(S2Smem<B>{stg}, S2Smem<B>{A}, A, tws, NoHook{});
-        const float ky = kf * (float)(iy < half ? iy : iy - N);
-        const float kz = kf * (float)(col0 + c);
-        const float kyz2 = ky * ky + kz * kz;
+        spass2<N, T, B, Q::F0, 1, -1, false>(S2Smem<B>{stg}, S2Smem<B>{A}, tws);
+        __syncthreads();
+        spass2<N, T, B, Q::F1, Q::F0, -1, true>(S2Smem<B>{A}, S2Smem<B>{A}, tws);
+        __syncthreads();
+        {
+            float2 p0[R], p1[R];
+            S2Smem<B>{A}.template load<R, LS>(l2, j, p0, p1);
+            __syncthreads();  // A has been read, it takes Psi below
 #pragma unroll
-        for (int q = 0; q < EPT; ++q) {
-            const int i = i0 + q * TB;
-            const float kx = kf * (float)(i < half ? i : i - N);
-            const float k2 = kx * kx + kyz2;
-            float gk = k2 > 0.f ? gscale / k2 : 0.f;
-            if (filt) {
-                // radial transfer T(|k|), piecewise linear on nodes b * fstep
-                const float u = sqrtf(k2) / fstep;
-                int b = (int)u;
-                if (b > nfilt - 2) b = nfilt - 2;
-                const float f = fminf(u - (float)b, 1.f);
-                gk *= (1.f - f) * filt[b] + f * filt[b + 1];
+            for (int r = 1; r < R; ++r) {
+                const float2 w = tws[r * j];
+                p0[r] = cmul(p0[r], w);
+                p1[r] = cmul(p1[r], w);
             }
-            float2& x = elem(A, q);
-            x = cscale(x, gk);
+            SmallDft<R>::run(p0, -1);
+            SmallDft<R>::run(p1, -1);
+            const float ky = kf * (float)(iy < half ? iy : iy - N);
+            const float kz0 = kf * (float)(col0 + 2 * l2), kz1 = kf * (float)(col0 + 2 * l2 + 1);
+            const float kyz0 = ky * ky + kz0 * kz0, kyz1 = ky * ky + kz1 * kz1;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = j + r * LS;
+                const float kx = kf * (float)(i < half ? i : i - N);
+                const float ka = kx * kx + kyz0, kb = kx * kx + kyz1;
+                float g0 = ka > 0.f ? gscale / ka : 0.f, g1 = kb > 0.f ? gscale / kb : 0.f;
+                if (filt) {
+                    g0 *= radial_filter(ka, filt, nfilt, fstep);
+                    g1 *= radial_filter(kb, filt, nfilt, fstep);
+                }
+                p0[r] = cscale(p0[r], g0);
+                p1[r] = cscale(p1[r], g1);
+            }
+            float2 u0[R], u1[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = j + r * LS;
+                const float kx = (i == half) ? 0.f : kf * (float)(i < half ? i : i - N);
+                u0[r] = make_float2(-kx * p0[r].y, kx * p0[r].x);  // i k_x phi
+                u1[r] = make_float2(-kx * p1[r].y, kx * p1[r].x);
+            }
+            SmallDft<R>::run(u0, +1);
+            SmallDft<R>::run(u1, +1);
+            S2Smem<B>{stg}.template store<R, 1>(l2, j * R, u0, u1);
+            SmallDft<R>::run(p0, +1);
+            SmallDft<R>::run(p1, +1);
+            S2Smem<B>{A}.template store<R, 1>(l2, j * R, p0, p1);
         }
         __syncthreads();
-        sip2_run<N, T, B, +1, false, false, typename GreenPlans<N>::I1>(Ikx2Load<N, B>{A, kf}, SX2IO<N>{F + off}, stg,
-                                                                        tws, NoHook{});
+        spass2<N, T, B, Q::I1, R, +1, true>(S2Smem<B>{stg}, S2Smem<B>{stg}, tws);
+        __syncthreads();
+        spass2<N, T, B, Q::I2, R * Q::I1, +1, false>(S2Smem<B>{stg}, SX2IO<N>{F + off}, tws);
+        __syncthreads();
         const int tn = t + gridDim.x;
         if (tn < ntiles) stile_prefetch<N, B, T>(stg, F + tile_off(tn), xo);
-        sip2_run<N, T, B, +1, true, false, typename GreenPlans<N>::I2>(S2Smem<B>{A}, SX2IO<N>{F + off + G::P}, A,
-                                                                       tws, NoHook{});
+        spass2<N, T, B, Q::I1, R, +1, true>(S2Smem<B>{A}, S2Smem<B>{A}, tws);
+        __syncthreads();
+        spass2<N, T, B, Q::I2, R * Q::I1, +1, false>(S2Smem<B>{A}, SX2IO<N>{F + off + G::P}, tws);
     }
 }
 
@@ -1114,6 +1150,20 @@ struct FixStage {
 
 // entries of the pass-ordered twiddle table of an M-point plan
 constexpr int ordered_tw_size(int M) { return tw_offset(static_plan(M), static_plan(M).nr); }
+
+// Radix order of the warp-row r2c + deposit: the butterflies of a pass spread
+// evenly over 32 lanes where the line allows it (768 = 24 8 4: 1, 3 and 6 rounds
+// without an idle lane, against 2, 2 and 6 with 16 12 4; the pass at 1536 took 13.0
+// ms instead of 15.4).  The c2r + gather keeps the default order: at 80 registers
+// the 24 values in flight spill (21.0 ms against 18.4).
+template <int M>
+struct WarpPlan : PlanOf<M> {};
+template <>
+struct WarpPlan<768> : PlanOf<768, 24, 8, 4> {};
+template <int M>
+constexpr int warp_tw_size() {
+    return tw_offset(WarpPlan<M>::P, WarpPlan<M>::P.nr);
+}
 
 // c2r pre-processing read straight from a row X[0..M] in global memory (the
 // same arithmetic as C2rStage)
