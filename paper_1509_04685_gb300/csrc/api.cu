@@ -322,12 +322,12 @@ static int power_common(const cola_config* cfg, const cola_state* st, int32_t no
                                 status_ptr(ws), s, rsd)))
         return rc;
     const long long Ppk = fft_pitch(ng_pk);
+    const int xbs = pk_xbs(ng_pk);
     if ((rc = fft_z_r2c(dep, mk, ng_pk, (float)(ratio * ratio * ratio / 1099511627776.0), tw, s, Ppk,
-                        (long long)ng_pk * ng_pk, FRow{ng_pk, 0, 1}, false)))
+                        (long long)ng_pk * ng_pk, FRow{ng_pk, xbs, 1}, false)))
         return rc;
-    if ((rc = fft_strided(mk, ng_pk, 1, -1, tw, s))) return rc;
-    if ((rc = fft_strided(mk, ng_pk, 0, -1, tw, s))) return rc;
-    return launch_power(mk, ng_pk, Ppk, cfg->box, flags, reinterpret_cast<double*>(wsp(ws, L.pk_part)),
+    if ((rc = fft_xy_forward(mk, ng_pk, xbs, tw, s))) return rc;
+    return launch_power(mk, ng_pk, xbs, Ppk, cfg->box, flags, reinterpret_cast<double*>(wsp(ws, L.pk_part)),
                         reinterpret_cast<float*>(dep), k, pk, nmodes, nbins, s, p2, p4);
 }
 

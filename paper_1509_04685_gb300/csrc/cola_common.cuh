@@ -606,6 +606,11 @@ int fft_z_c2r(float2* data, int n, const float2* tw, cudaStream_t s, float* out,
 int fft_lines(float2* data, int n, int sign, const float2* tw, cudaStream_t s, LineGeom lg, int kid);
 // plain n x n x P mesh, axis 1 = y, 0 = x
 int fft_strided(float2* data, int n, int axis, int sign, const float2* tw, cudaStream_t s);
+// One-component mesh of the estimator: rows blocked by 2^pk_xbs(n) in x (three where
+// the x pass has a blocked form, else 0, the plain mesh), rows frow(x, y, 0, {n, xbs, 1});
+// fft_xy_forward: its forward y and x passes
+int pk_xbs(int n);
+int fft_xy_forward(float2* data, int n, int xbs, const float2* tw, cudaStream_t s);
 // interleaved force mesh (rows (ix, iy, c)): delta_k in c = 0 -> F_x, F_y, F_z in c = 0, 1, 2
 // filt: optional radial transfer function T(|k|) on nodes b * fstep, b < nfilt (nullptr: none)
 int fft_x_green(float2* F, int n, float gscale, float kf, const float2* tw, cudaStream_t s,
@@ -683,9 +688,10 @@ int launch_tables(const cola_config* cfg, double* table, double* scratch, cudaSt
 int launch_snapshot_coeffs(const cola_config* cfg, double a_node, double a_out, double* snap, double* scratch,
                            cudaStream_t s);
 int launch_ic(const cola_config* cfg, uint64_t seed, cola_state st, void* ws, const Layout& L, cudaStream_t s);
+// mk: rows frow(x, y, 0, {ng, xbs, 1}) of rs complex;
 // p2, p4 (optional, both or neither): quadrupole and hexadecapole about the z axis;
 // ctab: scratch of 8 ng^3 bytes (tables of the iterated Jing correction)
-int launch_power(const float2* mk, int ng, long long rs, double box, int flags, double* part, float* ctab, double* k,
+int launch_power(const float2* mk, int ng, int xbs, long long rs, double box, int flags, double* part, float* ctab, double* k,
                  double* pk, double* nmodes, int nbins, cudaStream_t s, double* p2 = nullptr, double* p4 = nullptr);
 size_t power_partial_bytes(int nbins);
 

@@ -51,13 +51,14 @@ int launch_twiddles(float2* tw, int n, cudaStream_t s) {
 // accessors for the z (row) passes.  Line l of a block is mesh row row0 + l.
 // ---------------------------------------------------------------------------
 // fixed-point CIC counts (2^40 per particle) -> delta = count*scale - 1, packed
-// as complex pairs; every count is cleared after it is read (with `clear`).
+// as complex pairs; every count is cleared after it is read with CLEAR (a
+// run-time flag made the 16-row first pass slower: step 320^3 on 640^3 12.4 ms for 11.6).
+template <bool CLEAR>
 struct FixRowLoader {
     unsigned long long* dep;
     int n;
     long long row0, nrows;
     float scale;
-    bool clear;
     template <int R>
     __device__ __forceinline__ void load(int l, int i0, int di, float2* v) const {
         const long long row = row0 + l;
@@ -73,7 +74,7 @@ struct FixRowLoader {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             v[r] = make_float2((float)c[r].x * scale - 1.0f, (float)c[r].y * scale - 1.0f);
-            if (clear) __stcs(p + i0 + r * di, make_ulonglong2(0ull, 0ull));
+            if (CLEAR) __stcs(p + i0 + r * di, make_ulonglong2(0ull, 0ull));
         }
     }
 };
@@ -234,10 +235,10 @@ struct YZStore {
 // A real row is packed as n/2 complex values, transformed, and unpacked with
 // X[k] = E[k] + W^k O[k], E = (Z[k] + conj Z[M-k])/2, O = (Z[k] - conj Z[M-k])/(2i).
 // ---------------------------------------------------------------------------
-template <bool FIX>
+template <bool FIX, bool CLEAR>
 __global__ void k_fft_z_r2c(unsigned long long* __restrict__ dep, float2* out, int n, long long rs, long long nrows,
                             int NR, float scale, FftPlan plan, const float2* __restrict__ tw, FastDiv m1div, FRow fr,
-                            bool clear, int* clean) {
+                            int* clean) {
     if (clean && blockIdx.x == 0 && threadIdx.x == 0) *clean = kDepClean;
     extern __shared__ float2 sm[];
     __shared__ long long obase[64];  // output row offsets of this block's lines
@@ -253,7 +254,7 @@ __global__ void k_fft_z_r2c(unsigned long long* __restrict__ dep, float2* out, i
     const FftGeom g{NR, ls, 1, false, 0, 2};
     const float2* Z;
     if (FIX)
-        Z = fft_run_smem<-1, false>(FixRowLoader{dep, n, row0, nrows, scale, clear}, sm, sb, plan, g, tw);
+        Z = fft_run_smem<-1, false>(FixRowLoader<CLEAR>{dep, n, row0, nrows, scale}, sm, sb, plan, g, tw);
     else
         Z = fft_run_smem<-1, false>(RowLoader{out, rs, row0, nrows}, sm, sb, plan, g, tw);
     for (int e = threadIdx.x; e < NR * (M + 1); e += blockDim.x) {
@@ -493,15 +494,10 @@ int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const fl
     ProfScope ps(dep ? kKZr2cFix : kKZr2c, s);
     int rc = COLA_OK;
     if (dep && launch_z_r2c_fix_static(dep, out, n, rs, nrows, scale, tw, fr, clear, clean, s, &rc)) return rc;
-    if (dep) {
-        if (!set_smem((const void*)k_fft_z_r2c<true>, smem)) return COLA_ECUDA;
-        k_fft_z_r2c<true><<<(unsigned)grid, T, smem, s>>>(dep, out, n, rs, nrows, NR, scale, plan, tw,
-                                                           make_fastdiv(M + 1), fr, clear, clean);
-    } else {
-        if (!set_smem((const void*)k_fft_z_r2c<false>, smem)) return COLA_ECUDA;
-        k_fft_z_r2c<false><<<(unsigned)grid, T, smem, s>>>(nullptr, out, n, rs, nrows, NR, 0.f, plan, tw,
-                                                            make_fastdiv(M + 1), fr, false, nullptr);
-    }
+    auto kern = !dep ? k_fft_z_r2c<false, false> : (clear ? k_fft_z_r2c<true, true> : k_fft_z_r2c<true, false>);
+    if (!set_smem((const void*)kern, smem)) return COLA_ECUDA;
+    kern<<<(unsigned)grid, T, smem, s>>>(dep, out, n, rs, nrows, NR, dep ? scale : 0.f, plan, tw, make_fastdiv(M + 1), fr,
+                                         clean);
     return check_launch();
 }
 
@@ -716,6 +712,22 @@ int fft_strided(float2* data, int n, int axis, int sign, const float2* tw, cudaS
     const LineGeom lg = axis == 1 ? LineGeom{P, n, 1, (long long)n * P, 0} : LineGeom{(long long)n * P, n, 1, P, 0};
     return fft_lines(data, n, sign, tw, s, lg,
                      axis == 1 ? (sign < 0 ? kKYFwd : kKYInv) : (sign < 0 ? kKXFwd : kKXInv));
+}
+
+int pk_xbs(int n) { return blocked_x_static(n, strided_cols(n)) ? 3 : 0; }
+
+int fft_xy_forward(float2* data, int n, int xbs, const float2* tw, cudaStream_t s) {
+    int rc;
+    if (xbs == 0) {
+        if ((rc = fft_strided(data, n, 1, -1, tw, s))) return rc;
+        return fft_strided(data, n, 0, -1, tw, s);
+    }
+    const long long P = fft_pitch(n), XB = 1ll << xbs;
+    if ((rc = fft_lines(data, n, -1, tw, s, LineGeom{XB * P, n, (int)XB, XB * n * P, P}, kKYFwd))) return rc;
+    const int B = strided_cols(n), nct = (n / 2 + 1 + B - 1) / B;
+    ProfScope ps(kKXFwd, s);
+    if (!launch_blocked_x_static(data, n, B, nct, n * nct, tw, s, &rc)) return COLA_EUNSUPPORTED_SIZE;
+    return rc;
 }
 
 int fft_x_green(float2* F, int n, float gscale, float kf, const float2* tw, cudaStream_t s, const float* filt,

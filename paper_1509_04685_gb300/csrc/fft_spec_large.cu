@@ -59,6 +59,34 @@ bool launch_strided_static(float2* data, int n, int B, int sign, LineGeom lg, in
     return launch_strided_static_small(data, n, B, sign, lg, nct, ntiles, tw, s, rc);
 }
 
+// (n, B, threads) of the x passes over a blocked one-component mesh
+#define COLA_XLINES_SPECS(X) \
+    X(768, 16, 512)          \
+    X(1024, 8, 256)          \
+    X(1152, 8, 384)          \
+    X(1536, 8, 384)          \
+    X(2304, 4, 384)
+
+bool blocked_x_static(int n, int B) {
+#define COLA_CASE(NN, BB, TT) \
+    if (n == NN && B == BB) return true;
+    COLA_XLINES_SPECS(COLA_CASE)
+#undef COLA_CASE
+    return false;
+}
+
+bool launch_blocked_x_static(float2* data, int n, int B, int nct, int ntiles, const float2* tw, cudaStream_t s,
+                             int* rc) {
+#define COLA_CASE(NN, BB, TT)                                        \
+    if (n == NN && B == BB) {                                        \
+        *rc = run_xlines2<NN, BB, TT>(data, nct, ntiles, tw, s);     \
+        return true;                                                 \
+    }
+    COLA_XLINES_SPECS(COLA_CASE)
+#undef COLA_CASE
+    return false;
+}
+
 bool launch_x_green_static(float2* F, int n, int B, int nct, int ntiles, const float2* tw, float gscale,
                            float kf, const float* filt, int nfilt, float fstep, cudaStream_t s, int* rc) {
 #define COLA_CASE(NN, BB, TT)                                                                      \

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(64) k_pk_jing_low(float* __restrict__ clow, in
 // computations in flight cost more than the turns.)  ITER: a pass of the iterated correction, which only needs
 // the sums of w P (the counts and sums of w k do not change).
 template <bool MULTI, bool ITER>
-__global__ void __launch_bounds__(kPkThreads) k_pk_shells(const float2* __restrict__ mk, int ng, long long P,
+__global__ void __launch_bounds__(kPkThreads) k_pk_shells(const float2* __restrict__ mk, int ng, int xbs, long long P,
                                                           float amp_scale, float kf, int flags, int nbins,
                                                           double* __restrict__ part, const float* __restrict__ ctab,
                                                           int low) {
@@ -141,7 +141,8 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_shells(const float2* __restri
     const unsigned first = blockIdx.x * kPkThreads + threadIdx.x, stride = gridDim.x * kPkThreads;
     const unsigned dr = stride / H, dz = stride - dr * H, dx = dr / ng, dy = dr - dx * ng;
     int kz = (int)(first % H), iy = (int)(first / H % ng), ix = (int)(first / H / ng);
-    auto value = [&] { return ix < ng ? __ldg(mk + ((long long)ix * ng + iy) * P + kz) : make_float2(0.f, 0.f); };
+    const FRow fr{ng, xbs, 1};
+    auto value = [&] { return ix < ng ? __ldg(mk + frow(ix, iy, 0, fr) * P + kz) : make_float2(0.f, 0.f); };
     float2 next = value();
     while (ix < ng) {
         const float2 d = next;
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_shells(const float2* __restri
 // 1e4 in single bins, and that rounding depends on the order in which the warps
 // of a block reach its bins, hence on the pace of this loop; it stays as it is
 // so that iterated spectra stay as near to earlier ones as two runs are.
-__global__ void __launch_bounds__(kPkThreads) k_pk_shells_first(const float2* __restrict__ mk, int ng, long long P,
+__global__ void __launch_bounds__(kPkThreads) k_pk_shells_first(const float2* __restrict__ mk, int ng, int xbs, long long P,
                                                                 float amp_scale, float kf, int nbins,
                                                                 double* __restrict__ part) {
     extern __shared__ float bins[];
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(kPkThreads) k_pk_shells_first(const float2* __
         while ((long long)i * i + i < n2) ++i;
         while ((long long)i * i - i + 1 > n2) --i;
         if (i < 1 || i > nbins) continue;
-        const float2 d = mk[row * P + kz];
+        const float2 d = mk[frow(ix, iy, 0, FRow{ng, xbs, 1}) * P + kz];
         const float re = d.x * amp_scale, im = d.y * amp_scale;
         float p = __fmaf_rn(re, re, __fmul_rn(im, im));
         float W = 1.f, C = 1.f;
@@ -311,7 +312,7 @@ __global__ void k_pk_slopes(const double* __restrict__ k, const double* __restri
     }
 }
 
-int launch_power(const float2* mk, int ng, long long rs, double box, int flags, double* part, float* ctab, double* k,
+int launch_power(const float2* mk, int ng, int xbs, long long rs, double box, int flags, double* part, float* ctab, double* k,
                  double* pk, double* nmodes, int nbins, cudaStream_t s, double* p2, double* p4) {
     const double ng3 = (double)ng * ng * ng;
     const float amp_scale = (float)(box * sqrt(box) / ng3);  // sqrt(L^3 / ng^6)
@@ -334,7 +335,7 @@ int launch_power(const float2* mk, int ng, long long rs, double box, int flags, 
         if (!set_smem((const void*)kern, smem)) return COLA_ECUDA;
         {
             ProfScope ps(kKPkShells, s);
-            kern<<<kPkBlocks, kPkThreads, smem, s>>>(mk, ng, rs, amp_scale, kf, fl, nbins, part, ctab, low);
+            kern<<<kPkBlocks, kPkThreads, smem, s>>>(mk, ng, xbs, rs, amp_scale, kf, fl, nbins, part, ctab, low);
         }
         return reduce();
     };
@@ -342,7 +343,7 @@ int launch_power(const float2* mk, int ng, long long rs, double box, int flags, 
     // closed-form start, then kJingIterations passes with slopes from the last estimate
     {
         ProfScope ps(kKPkShells, s);
-        k_pk_shells_first<<<kPkBlocks, kPkThreads, 3 * (size_t)nbins * sizeof(float), s>>>(mk, ng, rs, amp_scale, kf,
+        k_pk_shells_first<<<kPkBlocks, kPkThreads, 3 * (size_t)nbins * sizeof(float), s>>>(mk, ng, xbs, rs, amp_scale, kf,
                                                                                         nbins, part);
     }
     int rc = reduce();
