@@ -496,8 +496,8 @@ int fft_z_r2c(unsigned long long* dep, float2* out, int n, float scale, const fl
     if (dep && launch_z_r2c_fix_static(dep, out, n, rs, nrows, scale, tw, fr, clear, clean, s, &rc)) return rc;
     auto kern = !dep ? k_fft_z_r2c<false, false> : (clear ? k_fft_z_r2c<true, true> : k_fft_z_r2c<true, false>);
     if (!set_smem((const void*)kern, smem)) return COLA_ECUDA;
-    kern<<<(unsigned)grid, T, smem, s>>>(dep, out, n, rs, nrows, NR, dep ? scale : 0.f, plan, tw, make_fastdiv(M + 1), fr,
-                                         clean);
+    kern<<<(unsigned)grid, T, smem, s>>>(dep, out, n, rs, nrows, NR, dep ? scale : 0.f, plan, tw, make_fastdiv(M + 1),
+                                         fr, clean);
     return check_launch();
 }
 

@@ -64,8 +64,7 @@ bool launch_strided_static(float2* data, int n, int B, int sign, LineGeom lg, in
     X(768, 16, 512)          \
     X(1024, 8, 256)          \
     X(1152, 8, 384)          \
-    X(1536, 8, 384)          \
-    X(2304, 4, 384)
+    X(1536, 8, 384)
 
 bool blocked_x_static(int n, int B) {
 #define COLA_CASE(NN, BB, TT) \
@@ -156,9 +155,9 @@ bool static_tile_ok(int n, int B) {
 
 // (n, warps per block, blocks per SM) of the warp-row r2c of the fixed-point
 // counts; it takes precedence.  At 1024 it takes 2.11 ms against 4.32 ms for the
-// block tile (8 warps per SM fit there, 32 here), at 512 0.50 against 0.51 ms.  (At 1152 it was slower than the block tile,
-// 6.6 ms against 5.8 ms, and a warp-row plain c2r was slower at 2304, 74 ms
-// against 64 ms.)
+// block tile (8 warps per SM fit there, 32 here), at 512 0.50 against 0.51 ms.
+// (At 1152 it was slower than the block tile, 6.6 ms against 5.8 ms, and a
+// warp-row plain c2r was slower at 2304, 74 ms against 64 ms.)
 #define COLA_ZWARP_SPECS(X) \
     X(512, 16, 2)           \
     X(1024, 16, 2)          \

@@ -17,8 +17,9 @@
 // chain that is left is one map per time node.  The steps, the stages and the
 // formulas are those of the serial integration, one thread walking ~1400 steps
 // of four right-hand sides: 21.4 ms per table (40 nodes) and 18.8 ms per
-// snapshot that way, 77 and 61 us this way (two launches each).  What bounds it now is FP64 issue (about two lanes per
-// clock and SM), hence one warp per block, spread over the SMs.
+// snapshot that way, 0.15 ms and 61 us this way (two launches each).  What bounds
+// it now is FP64 issue (about two lanes per clock and SM), hence one warp per
+// block, spread over the SMs.
 #include <cmath>
 
 #include "cosmo.cuh"
@@ -392,7 +393,7 @@ __global__ void __launch_bounds__(kRowThreads) k_table_rows(double* tab, const d
                 o[4] = k / (kn * ajn * E_of(aj, c));
             }
         }
-        __syncthreads();  // every row of this round has been read
+        __syncthreads();  // every row of this batch has been read
         if (j < n) {
             double* r = tab + (size_t)j * kTableCols;
 #pragma unroll

@@ -62,3 +62,23 @@ def test_shell_sums_of_the_density(nq, ng):
         torch.testing.assert_close(kk, s[1] / s[0] * (2 * math.pi / L), rtol=2e-6, atol=0.0)
         torch.testing.assert_close(pp, s[2] / s[0], rtol=2e-5, atol=0.0)  # the P(k) parity tolerance
     torch.testing.assert_close(p2, 5 * s[3] / s[0], rtol=0.0, atol=1e-4 * float((s[2] / s[0]).max()))
+
+
+@pytest.mark.parametrize("ng", [768, 1024, 1152, 1536])
+def test_power_of_blocked_rows(ng):
+    # the blocked estimator mesh and its x pass against the plain mesh (four columns per tile)
+    nq, L = 64, 100.0
+    sim = C.Simulation(C.make_config(nq, ng, L, 0.05, 1.0, 40))
+    sim.init_tables()
+    g = torch.Generator(device="cuda").manual_seed(ng)
+    sim.d.copy_(torch.randn(sim.d.shape, generator=g, device="cuda") * 3.0)
+    k, p, n = sim.power(ng, a_out=0.05, node=0)
+    C.cola_fft_set_tile(ng, 4)
+    try:
+        k4, p4, n4 = sim.power(ng, a_out=0.05, node=0)
+    finally:
+        C.cola_fft_set_tile(ng, 0)
+    assert sim.status() == 0
+    assert torch.equal(n, n4)
+    torch.testing.assert_close(k, k4, rtol=2e-6, atol=0.0)
+    torch.testing.assert_close(p, p4, rtol=2e-5, atol=0.0)  # the P(k) parity tolerance
