@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "../../include/cola.h"
+#include "smem.h"
 
 namespace cola {
 
@@ -576,7 +577,6 @@ class ProfScope {
 // host-side launch helpers (defined in the .cu files)
 // ---------------------------------------------------------------------------
 extern unsigned long long g_launches;
-extern int g_last_cuda_error;  // the CUDA error behind the last COLA_ECUDA of a launch (cola_last_cuda_error)
 inline int check_launch() {
     g_launches++;
     const cudaError_t e = cudaGetLastError();
@@ -586,8 +586,6 @@ inline int check_launch() {
 }
 
 int launch_twiddles(float2* tw, int n, cudaStream_t s);
-// raise a kernel's dynamic shared-memory limit (cached per kernel and size)
-bool set_smem(const void* fn, size_t bytes);
 // persistent grid: blocks per SM from the shared-memory budget, at most ntiles
 int num_sms();  // of the current device (cached)
 int persistent_grid(size_t smem, int ntiles);

@@ -444,35 +444,6 @@ static int z_rows_per_block(int M) {
     return nr;
 }
 
-// Raise a kernel's dynamic shared-memory limit once per size (also keeps the
-// attribute call out of stream captures after the first, uncaptured use).
-bool set_smem(const void* fn, size_t bytes) {
-    // the 48 KB a launch may take without the attribute covers static and
-    // dynamic shared memory together; the kernels' static arrays stay far below 8 KB
-    if (bytes + 8 * 1024 <= 48 * 1024) return true;
-    static const void* fns[64];
-    static size_t done[64];
-    static int nf = 0;
-    for (int i = 0; i < nf; ++i)
-        if (fns[i] == fn && done[i] >= bytes) return true;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) {
-        g_last_cuda_error = (int)e;
-        cudaGetLastError();
-        return false;
-    }
-    for (int i = 0; i < nf; ++i)
-        if (fns[i] == fn) {
-            done[i] = bytes;
-            return true;
-        }
-    if (nf < 64) {
-        fns[nf] = fn;
-        done[nf++] = bytes;
-    }
-    return true;
-}
-
 // threads: about one butterfly of the first (largest-radix) pass per thread
 static int pass_threads(const FftPlan& plan, long lines) {
     long t = plan.n / plan.radix[0] * lines;
