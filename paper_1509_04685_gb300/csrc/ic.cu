@@ -6,6 +6,7 @@
 #include <cmath>
 
 #include "cosmo.cuh"
+#include "noise.cuh"
 
 namespace cola {
 
@@ -105,92 +106,8 @@ __global__ void __launch_bounds__(256) k_ic_amp(const double* __restrict__ part,
 }
 
 // ---------------------------------------------------------------------------
-// Philox-4x32-10 (Salmon et al. 2011) and the white-noise field
+// white-noise field (noise.cuh)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint4 philox4x32_10(uint4 ctr, uint2 key) {
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        if (r > 0) {
-            key.x += 0x9E3779B9u;
-            key.y += 0xBB67AE85u;
-        }
-        const unsigned lo0 = 0xD2511F53u * ctr.x, hi0 = __umulhi(0xD2511F53u, ctr.x);
-        const unsigned lo1 = 0xCD9E8D57u * ctr.z, hi1 = __umulhi(0xCD9E8D57u, ctr.z);
-        ctr = make_uint4(hi1 ^ ctr.y ^ key.x, lo1, hi0 ^ ctr.w ^ key.y, lo0);
-    }
-    return ctr;
-}
-
-// Box-Muller draw sqrt(-2 ln u1) cos(2 pi u2) with u = m 2^-53, m = (a >> 5) 2^26 +
-// (b >> 6) + 1 in [1, 2^53], in FP64.  The result is rounded to FP32, so series
-// that are good to 1e-11 do (the library's log, sqrt and cospi to the last of 53
-// bits took 70 FP64 instructions per cell and 1.87 ms at 256^3, bound by the two
-// FP64 lanes per clock of an SM; this takes about half).  Conversions and range
-// reductions are integer work:
-//   ln f for f in [sqrt(1/2), sqrt(2)) from the atanh series in s = (f - 1) / (f + 1),
-//   s^2 <= 0.0295, through s^15; quotient and root by one Newton step from an FP32
-//   seed; cos and sin of pi r, |r| <= 1/4, by their Taylor series through order 14.
-__device__ __forceinline__ float as_float(double x) {  // FP32 value near x, 1e-30 < x < 1e30, from the bits
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    return __uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29));
-}
-__device__ __forceinline__ double as_double(float x) {  // the FP32 value x > 0 (normal), from the bits
-    const unsigned u = __float_as_uint(x);
-    return __hiloint2double((int)((u >> 3) + (896u << 20)), (int)(u << 29));
-}
-
-__device__ __forceinline__ float box_muller(uint4 w) {
-    const double two52 = 4503599627370496.0;
-    // u1 2^53 and its logarithm
-    const double m1 = fma(__hiloint2double(0x43300000, (int)(w.x >> 5)) - two52, 67108864.0,
-                          __hiloint2double(0x43300000, (int)((w.y >> 6) + 1u)) - two52);
-    const int hi = __double2hiint(m1);
-    int e = (hi >> 20) - 1023 - 53;
-    int top = (hi & 0xfffff) | 0x3ff00000;
-    if (top >= 0x3ff6a09e) {  // f >= sqrt(2), to 20 bits: halve it
-        top -= 1 << 20;
-        ++e;
-    }
-    const double f = __hiloint2double(top, __double2loint(m1));
-    const double q = f + 1.0;
-    double rq = as_double(__frcp_rn(as_float(q)));
-    rq = fma(rq, fma(-q, rq, 1.0), rq);
-    const double s = (f - 1.0) * rq, z = s * s;
-    double p = 1.0 / 15.0;
-    p = fma(p, z, 1.0 / 13.0);
-    p = fma(p, z, 1.0 / 11.0);
-    p = fma(p, z, 1.0 / 9.0);
-    p = fma(p, z, 1.0 / 7.0);
-    p = fma(p, z, 1.0 / 5.0);
-    p = fma(p, z, 1.0 / 3.0);
-    p = fma(p * z, s, s);  // ln f = 2 p
-    const double ed = __hiloint2double(0x43300000, e + 0x400) - (two52 + 1024.0);  // e in [-53, 0]
-    const double x = fma(-4.0, p, ed * -1.3862943611198906188);                    // -2 ln u1
-    if (!(x > 0.0)) return 0.f;  // u1 = 1
-    const float seed = rsqrtf(as_float(x));
-    const double rs = as_double(seed);
-    double y = x * rs;
-    y = fma(fma(-y, y, x), 0.5 * rs, y);  // sqrt(x)
-    // cos(2 pi u2) = cos(pi m2 2^-52): k half turns of pi/2, remainder r 2^-52
-    const long long m2 = ((long long)(w.z >> 5) << 26) + (long long)(w.w >> 6) + 1;
-    const int k = (int)((m2 + (1ll << 50)) >> 51);
-    const long long rem = m2 - ((long long)k << 51);  // |rem| <= 2^50
-    const double r = __longlong_as_double(0x4338000000000000ll + rem) - 6755399441055744.0;
-    const double t = r * (3.14159265358979323846 / two52), u = t * t;
-    const bool odd = k & 1;  // sine of the remainder
-    double c = odd ? 1.0 / 6227020800.0 : -1.0 / 87178291200.0;
-    c = fma(c, u, odd ? -1.0 / 39916800.0 : 1.0 / 479001600.0);
-    c = fma(c, u, odd ? 1.0 / 362880.0 : -1.0 / 3628800.0);
-    c = fma(c, u, odd ? -1.0 / 5040.0 : 1.0 / 40320.0);
-    c = fma(c, u, odd ? 1.0 / 120.0 : -1.0 / 720.0);
-    c = fma(c, u, odd ? -1.0 / 6.0 : 1.0 / 24.0);
-    c = fma(c, u, odd ? 1.0 : -0.5);
-    c = odd ? c * t : fma(c, u, 1.0);
-    // k = 0, 4: cos; 1: -sin; 2: -cos; 3: sin
-    if (k == 1 || k == 2) c = -c;
-    return (float)(y * c);
-}
-
 // noise of Lagrangian cell (i, j, k) -> real view of an nq mesh (row pitch 2P floats)
 __global__ void k_noise(float* mesh, int nq, long long P2, unsigned long long seed) {
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -200,7 +117,7 @@ __global__ void k_noise(float* mesh, int nq, long long P2, unsigned long long se
                                   make_uint2((unsigned)seed, (unsigned)(seed >> 32)));
     const long long row = n / nq;
     const int k = (int)(n - row * nq);
-    mesh[row * P2 + k] = box_muller(w);
+    mesh[row * P2 + k] = (float)box_muller(w);
 }
 
 // ---------------------------------------------------------------------------
