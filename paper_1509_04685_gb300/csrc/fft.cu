@@ -685,7 +685,7 @@ int fft_strided(float2* data, int n, int axis, int sign, const float2* tw, cudaS
                      axis == 1 ? (sign < 0 ? kKYFwd : kKYInv) : (sign < 0 ? kKXFwd : kKXInv));
 }
 
-int pk_xbs(int n) { return blocked_x_static(n, strided_cols(n)) ? 3 : 0; }
+int pk_xbs(int n) { return strided_cols(n) == blocked_x_cols(n) ? 3 : 0; }
 
 int fft_xy_forward(float2* data, int n, int xbs, const float2* tw, cudaStream_t s) {
     int rc;
@@ -695,10 +695,8 @@ int fft_xy_forward(float2* data, int n, int xbs, const float2* tw, cudaStream_t 
     }
     const long long P = fft_pitch(n), XB = 1ll << xbs;
     if ((rc = fft_lines(data, n, -1, tw, s, LineGeom{XB * P, n, (int)XB, XB * n * P, P}, kKYFwd))) return rc;
-    const int B = strided_cols(n), nct = (n / 2 + 1 + B - 1) / B;
     ProfScope ps(kKXFwd, s);
-    if (!launch_blocked_x_static(data, n, B, nct, n * nct, tw, s, &rc)) return COLA_EUNSUPPORTED_SIZE;
-    return rc;
+    return launch_blocked_x_static(data, n, tw, s);
 }
 
 int fft_x_green(float2* F, int n, float gscale, float kf, const float2* tw, cudaStream_t s, const float* filt,

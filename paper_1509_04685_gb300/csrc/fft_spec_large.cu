@@ -66,24 +66,23 @@ bool launch_strided_static(float2* data, int n, int B, int sign, LineGeom lg, in
     X(1152, 8, 384)          \
     X(1536, 8, 384)
 
-bool blocked_x_static(int n, int B) {
+int blocked_x_cols(int n) {
 #define COLA_CASE(NN, BB, TT) \
-    if (n == NN && B == BB) return true;
+    if (n == NN) return BB;
     COLA_XLINES_SPECS(COLA_CASE)
 #undef COLA_CASE
-    return false;
+    return 0;
 }
 
-bool launch_blocked_x_static(float2* data, int n, int B, int nct, int ntiles, const float2* tw, cudaStream_t s,
-                             int* rc) {
+int launch_blocked_x_static(float2* data, int n, const float2* tw, cudaStream_t s) {
 #define COLA_CASE(NN, BB, TT)                                        \
-    if (n == NN && B == BB) {                                        \
-        *rc = run_xlines2<NN, BB, TT>(data, nct, ntiles, tw, s);     \
-        return true;                                                 \
+    if (n == NN) {                                                   \
+        constexpr int nct = (NN / 2 + 1 + BB - 1) / BB;              \
+        return run_xlines2<NN, BB, TT>(data, nct, NN * nct, tw, s);  \
     }
     COLA_XLINES_SPECS(COLA_CASE)
 #undef COLA_CASE
-    return false;
+    return COLA_EUNSUPPORTED_SIZE;
 }
 
 bool launch_x_green_static(float2* F, int n, int B, int nct, int ntiles, const float2* tw, float gscale,

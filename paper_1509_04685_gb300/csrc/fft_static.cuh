@@ -1465,10 +1465,11 @@ bool launch_strided_static(float2* data, int n, int B, int sign, LineGeom lg, in
                            const float2* tw, cudaStream_t s, int* rc);
 bool launch_x_green_static(float2* F, int n, int B, int nct, int ntiles, const float2* tw, float gscale, float kf,
                            const float* filt, int nfilt, float fstep, cudaStream_t s, int* rc);
-// forward x pass of a one-component mesh blocked by eight in x, where it pays
-// (blocked_x_static); false without a specialisation of (n, B)
-bool blocked_x_static(int n, int B);
-bool launch_blocked_x_static(float2* data, int n, int B, int nct, int ntiles, const float2* tw, cudaStream_t s, int* rc);
+// forward x pass of a one-component mesh blocked by eight in x, where it pays: its
+// column width (0: no such pass), which does not depend on the width the other
+// passes use, so a mesh laid out for it can be transformed whatever that is by then
+int blocked_x_cols(int n);
+int launch_blocked_x_static(float2* data, int n, const float2* tw, cudaStream_t s);
 // z passes of the step: the in-place c2r of the force rows and the r2c of the
 // fixed-point counts (fft_spec_large.cu)
 bool launch_z_c2r_static(float2* data, int n, long long rs, long long nrows, const float2* tw, cudaStream_t s,
