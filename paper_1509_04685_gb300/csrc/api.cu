@@ -305,7 +305,7 @@ static int power_common(const cola_config* cfg, const cola_state* st, int32_t no
     const double a_node = host_node_a(cfg, node);
     const double* snap = nullptr;
     if (rsd || std::fabs(a_out - a_node) > 1e-12 * a_node) {
-        if (!(a_out > 0.0) || !state_ok(st, true)) return COLA_EINVAL;
+        if (!(a_out > 0.0) || !std::isfinite(a_out) || !state_ok(st, true)) return COLA_EINVAL;
         double* sp = reinterpret_cast<double*>(wsp(ws, kHdrSnap));
         if ((rc = launch_snapshot_coeffs(cfg, a_node, a_out, sp, growth_ptr(ws), s))) return rc;
         snap = sp;
