@@ -16,7 +16,12 @@ static int check_config(const cola_config* c) {
         return COLA_EINVAL;
     if (c->n_steps < 2 || c->n_steps > kMaxSteps) return COLA_EINVAL;
     if (c->sampling < COLA_SAMPLING_LINEAR || c->sampling > COLA_SAMPLING_POW) return COLA_EINVAL;
-    if (c->sampling == COLA_SAMPLING_POW && !(c->sampling_p > 0.0)) return COLA_EINVAL;
+    if (c->sampling == COLA_SAMPLING_POW) {
+        if (!(c->sampling_p > 0.0)) return COLA_EINVAL;
+        // a_init^p must not underflow: the first node would be a = 0 and the span from
+        // ln 0 of infinitely many steps (five units above zero cover pow's rounding)
+        if (!(std::pow(c->a_init, c->sampling_p) > 2.5e-323)) return COLA_EINVAL;
+    }
     const cola_cosmology& k = c->cosmo;
     if (!(k.omega_m > 0.0) || !(k.h > 0.0) || !(k.sigma8 > 0.0) || !(k.omega_b >= 0.0) || !(k.t_cmb > 0.0))
         return COLA_EINVAL;
