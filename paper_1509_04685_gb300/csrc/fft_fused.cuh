@@ -172,7 +172,9 @@ __device__ __forceinline__ void deposit_one(const TilePart& t, const int* bxy, i
 // the 64-bit weights gone as well, the whole pass took 15.4 ms instead of 18.8
 // (512^3 on 1536^3), 1.67 instead of 2.16 (256^3 on 768^3).  hi is at most 2^20
 // and |lo| 2^19 per particle, so the counters hold kSplitMax particles per cell;
-// tiles with more particles than that take deposit_one.
+// tiles with more particles than that take deposit_one.  (The tile's total bounds
+// any cell's count from above.  At nq = ng a tile of 16 rows lists 34 bins of nq
+// particles on average, 4352 at 128, so such meshes count in 64 bits.)
 constexpr int kSplitMax = 4095;
 __device__ __forceinline__ void deposit_one_split(const TilePart& t, const int* bxy, int ng, int x, int y0, int ty,
                                                   int* cnt) {

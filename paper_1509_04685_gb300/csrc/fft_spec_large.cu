@@ -114,7 +114,7 @@ static const int kGreenTiles[][2] = {{1152, 8}, {1536, 8}, {2304, 4}};
 int static_green_tile(int n) {
     for (const auto& e : kGreenTiles)
         if (e[0] == n) return e[1];
-    return launch_static_green_tile_small(n);
+    return 0;
 }
 
 int static_tile(int n) {
@@ -211,7 +211,9 @@ bool launch_z_r2c_fix_static(unsigned long long* dep, float2* out, int n, long l
 // (n, rows per tile, threads, blocks per SM) of the fused r2c + deposit pass.  The
 // meshes below 256 are those of the learned net, which takes this pass at any
 // size: at 128 the runtime form took 389 us, tiles of 32 rows (512 tiles for 456
-// resident blocks) 305, of 16 rows 203.
+// resident blocks) 305, of 16 rows 203.  With a particle per cell their tiles mostly
+// hold more than kSplitMax particles and count in 64 bits: the gain there is that
+// of the compile-time pass, not of the split counters.
 #define COLA_ZR2CD_SPECS(X) \
     X(64, 16, 128, 6)       \
     X(96, 16, 128, 6)       \

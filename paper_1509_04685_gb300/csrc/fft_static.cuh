@@ -382,16 +382,6 @@ struct IkxLoad {
     }
 };
 
-// Radix orders of the two-buffer fused pass's transforms (forward, F_x, Psi).
-// In-place passes may hold at most N B / T values per thread; a radix whose
-// butterflies do not spread evenly over the threads goes where its pass is out
-// of place (the forward's and F_x's first pass, Psi's last).
-template <int N>
-struct GreenPlans {
-    using F = PlanOf<N>;
-    using I1 = PlanOf<N>;
-    using I2 = PlanOf<N>;
-};
 // strided complex pass (y: S = row stride, outer = x; or x on a plain mesh):
 // persistent blocks; the first pass reads the staged tile into the working
 // buffer, after which the next tile is staged with cp.async while the other
@@ -478,8 +468,7 @@ __global__ void __launch_bounds__(T, 1) k_fft_x_green_s(float2* F, int nct, int 
         const long long off = (long long)iy * G::RS + col0;
         cp_async_wait_all();
         __syncthreads();
-        sip_run<N, T, Geo, -1, false, true, typename GreenPlans<N>::F>(SSmem<Geo>{stg}, SSmem<Geo>{A}, A, tws,
-                                                                      NoHook{});
+        sip_run<N, T, Geo, -1, false, true>(SSmem<Geo>{stg}, SSmem<Geo>{A}, A, tws, NoHook{});
         const float ky = kf * (float)(iy < half ? iy : iy - N);
         const float kz = kf * (float)(col0 + c);
         const float kyz2 = ky * ky + kz * kz;
@@ -494,12 +483,10 @@ __global__ void __launch_bounds__(T, 1) k_fft_x_green_s(float2* F, int nct, int 
             x = cscale(x, gk);
         }
         __syncthreads();
-        sip_run<N, T, Geo, +1, false, false, typename GreenPlans<N>::I1>(IkxLoad<N, Geo>{A, kf}, SXIO<N>{F + off}, stg,
-                                                                         tws, NoHook{});
+        sip_run<N, T, Geo, +1, false, false>(IkxLoad<N, Geo>{A, kf}, SXIO<N>{F + off}, stg, tws, NoHook{});
         const int tn = t + gridDim.x;
         if (tn < ntiles) stile_prefetch<N, B, T>(stg, F + tile_off(tn), xo);
-        sip_run<N, T, Geo, +1, true, false, typename GreenPlans<N>::I2>(SSmem<Geo>{A}, SXIO<N>{F + off + G::P}, A,
-                                                                        tws, NoHook{});
+        sip_run<N, T, Geo, +1, true, false>(SSmem<Geo>{A}, SXIO<N>{F + off + G::P}, A, tws, NoHook{});
     }
 }
 
@@ -1487,7 +1474,6 @@ bool static_tile_ok(int n, int B);
 // default column width of the specialised fused x/Green pass for n (0: the
 // strided passes' width)
 int static_green_tile(int n);
-int launch_static_green_tile_small(int n);
 // inverse y pass of the Psi component (k_fft_y_psi_s) for (n, B); false when
 // there is no specialisation, without launching
 bool launch_y_psi_static(float2* data, int n, int B, LineGeom lg, long long comp2, long long comp0, int nct,
