@@ -21,8 +21,11 @@
 // after the first two steps one load per pair shows for most of them, and
 // particles without a smaller friend are done before it.  (Uniting every pair
 // with two finds over particle-indexed parents took 23.0 ms at 512^3, the hook
-// and the link take 4.9 ms each; both wait on the loads of their candidates.)  Roots only ever hook
-// under smaller slots, in lock-free steps; a group's label is the smallest
+// and the link take 4.9 ms each; both wait on the loads of their candidates.)
+// Where hardly any particle has a friend the passes over the parents are what the
+// call takes more than that form did: at 512^3, L = 1536, node 3, b = 0.2, 7.24 ms
+// in both, and at 64^3, L = 192 0.095 ms for 0.083, four launches more.  Roots only
+// ever hook under smaller slots, in lock-free steps; a group's label is the smallest
 // particle index in it, so the labels do not depend on the order of anything.
 #include "cola_common.cuh"
 
@@ -221,20 +224,30 @@ __global__ void __launch_bounds__(256) k_fof_hook(const float4* __restrict__ sor
     parent[k] = first;
 }
 
-// every parent becomes (at least) the root its tree has now
+// every parent becomes (at least) the root its tree has now; four slots per
+// thread (np is a multiple of eight), as most parents are roots already in a
+// hardly clustered state and the pass is then one read of the parents
 __global__ void __launch_bounds__(256) k_fof_compress(int* parent, int np, int* status, int cap) {
-    const unsigned k = blockIdx.x * 256u + threadIdx.x;
-    if (k >= (unsigned)np) return;
-    int x = (int)k;
-    for (int it = 0; it < cap; ++it) {
-        const int px = __ldcg(parent + x);
-        if (px == x) {
-            if (x != (int)k) parent[k] = x;
-            return;
+    const unsigned k0 = (blockIdx.x * 256u + threadIdx.x) * 4u;
+    if (k0 >= (unsigned)np) return;
+    const int4 v = __ldcg(reinterpret_cast<const int4*>(parent + k0));
+    const int first[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int k = (int)k0 + q;
+        int x = first[q];
+        if (x == k) continue;
+        int it = 1;
+        for (; it < cap; ++it) {
+            const int px = __ldcg(parent + x);
+            if (px == x) break;
+            x = px;
         }
-        x = px;
+        if (it >= cap)
+            set_status(status, COLA_ETIMEOUT);
+        else if (x != first[q])
+            parent[k] = x;
     }
-    set_status(status, COLA_ETIMEOUT);
 }
 
 __global__ void __launch_bounds__(256) k_fof_link(const float4* __restrict__ sorted, const int* __restrict__ start,
@@ -270,18 +283,20 @@ __global__ void __launch_bounds__(256) k_fof_roots(const float4* __restrict__ so
     set_status(status, COLA_ETIMEOUT);
 }
 
-// least[root] = the smallest particle index of the group; a warp of one group takes one atomic
-__global__ void __launch_bounds__(256) k_fof_least(const float4* __restrict__ sorted, const int* __restrict__ parent,
-                                                   int np, int* least) {
+// least[root] = the smallest particle index of the group; a warp of one group takes
+// one atomic.  least[k] is the particle of slot k unless k is a root, whose own index
+// is in least[root] already, so neither needs the sorted records.
+__global__ void __launch_bounds__(256) k_fof_least(const int* __restrict__ parent, int np, int* least) {
     const unsigned k = blockIdx.x * 256u + threadIdx.x;
     const bool in = k < (unsigned)np;
     const int root = in ? __ldg(parent + k) : -1;
-    const int p = in ? __float_as_int(__ldg(&sorted[k].w)) : 0x7fffffff;
+    const bool adds = in && root != (int)k;
+    const int p = adds ? __ldcg(least + k) : 0x7fffffff;
     const unsigned full = 0xffffffffu;
     if (__all_sync(full, root == __shfl_sync(full, root, 0))) {
         const int m = __reduce_min_sync(full, p);
         if ((threadIdx.x & 31) == 0 && root >= 0) atomicMin(least + root, m);
-    } else if (in && root != (int)k) {
+    } else if (adds) {
         atomicMin(least + root, p);
     }
 }
@@ -397,10 +412,10 @@ int cola_fof(const cola_config* cfg, const cola_state* st, double b, int32_t* gr
     const int n = (int)np, nq = cfg->nq, cap = g_union_cap;
     const float b2 = (float)(b * b), reach = (float)b + 0.01f;  // wider than b by far more than FP32 rounding
     k_fof_hook<<<nb, T, 0, s>>>(sorted, start, n, nq, b2, reach, parent);
-    k_fof_compress<<<nb, T, 0, s>>>(parent, n, status, cap);
+    k_fof_compress<<<blocks_for(np, 4 * T), T, 0, s>>>(parent, n, status, cap);
     k_fof_link<<<nb, T, 0, s>>>(sorted, start, n, nq, b2, reach, parent, status, cap);
     k_fof_roots<<<nb, T, 0, s>>>(sorted, parent, n, least, status, cap);
-    k_fof_least<<<nb, T, 0, s>>>(sorted, parent, n, least);
+    k_fof_least<<<nb, T, 0, s>>>(parent, n, least);
     k_fof_label<<<nb, T, 0, s>>>(sorted, parent, least, n, group);
     if (int rc = check_launch()) return rc;
     return read_status(status, s);
