@@ -22,9 +22,11 @@
 // particles without a smaller friend are done before it.  (Uniting every pair
 // with two finds over particle-indexed parents took 23.0 ms at 512^3, the hook
 // and the link take 4.9 ms each; both wait on the loads of their candidates.)
-// Where hardly any particle has a friend the passes over the parents are what the
-// call takes more than that form did: at 512^3, L = 1536, node 3, b = 0.2, 7.24 ms
-// in both, and at 64^3, L = 192 0.095 ms for 0.083, four launches more.  Roots only
+// Where hardly any particle has a friend, hook and link find little to do and the
+// passes over the parents count: the particle of a slot is kept apart from the record
+// for them (512^3, L = 1536, node 3, b = 0.1: 6.75 ms for 6.70 in that form, b = 0.2:
+// 7.14 for 7.30).  Calls of up to 64^3 such particles pay for three launches more
+// (81 us for 65 at 32^3, 82 for 75 at 64^3; clustered ones take half the time).  Roots only
 // ever hook under smaller slots, in lock-free steps; a group's label is the smallest
 // particle index in it, so the labels do not depend on the order of anything.
 #include "cola_common.cuh"
@@ -209,9 +211,11 @@ __device__ __forceinline__ void smaller_friends(const float4* __restrict__ sorte
 
 __device__ __forceinline__ bool finite_pos(const float4& a) { return a.x == a.x && a.y == a.y && a.z == a.z; }
 
-// parent = the first friend below, or itself (non-finite input links to nothing)
+// parent = the first friend below, or itself (non-finite input links to nothing);
+// part[k] = the particle of slot k, so that k_fof_roots need not read the records again
 __global__ void __launch_bounds__(256) k_fof_hook(const float4* __restrict__ sorted, const int* __restrict__ start,
-                                                  int np, int nq, float b2, float reach, int* __restrict__ parent) {
+                                                  int np, int nq, float b2, float reach, int* __restrict__ parent,
+                                                  int* __restrict__ part) {
     const unsigned k = blockIdx.x * 256u + threadIdx.x;
     if (k >= (unsigned)np) return;
     const float4 a = __ldg(sorted + k);
@@ -222,6 +226,7 @@ __global__ void __launch_bounds__(256) k_fof_hook(const float4* __restrict__ sor
             return true;
         });
     parent[k] = first;
+    part[k] = __float_as_int(a.w);
 }
 
 // every parent becomes (at least) the root its tree has now; four slots per
@@ -266,11 +271,11 @@ __global__ void __launch_bounds__(256) k_fof_link(const float4* __restrict__ sor
 }
 
 // root of every slot; least[k] = the slot's particle, to be lowered by k_fof_least
-__global__ void __launch_bounds__(256) k_fof_roots(const float4* __restrict__ sorted, int* parent, int np,
+__global__ void __launch_bounds__(256) k_fof_roots(const int* __restrict__ part, int* parent, int np,
                                                    int* __restrict__ least, int* status, int cap) {
     const unsigned k = blockIdx.x * 256u + threadIdx.x;
     if (k >= (unsigned)np) return;
-    least[k] = __float_as_int(__ldg(&sorted[k].w));
+    least[k] = __ldg(part + k);
     int x = (int)k;
     for (int it = 0; it < cap; ++it) {
         const int px = __ldcg(parent + x);
@@ -411,10 +416,10 @@ int cola_fof(const cola_config* cfg, const cola_state* st, double b, int32_t* gr
     int* least = start;
     const int n = (int)np, nq = cfg->nq, cap = g_union_cap;
     const float b2 = (float)(b * b), reach = (float)b + 0.01f;  // wider than b by far more than FP32 rounding
-    k_fof_hook<<<nb, T, 0, s>>>(sorted, start, n, nq, b2, reach, parent);
+    k_fof_hook<<<nb, T, 0, s>>>(sorted, start, n, nq, b2, reach, parent, group);  // (group: scratch until the labels)
     k_fof_compress<<<blocks_for(np, 4 * T), T, 0, s>>>(parent, n, status, cap);
     k_fof_link<<<nb, T, 0, s>>>(sorted, start, n, nq, b2, reach, parent, status, cap);
-    k_fof_roots<<<nb, T, 0, s>>>(sorted, parent, n, least, status, cap);
+    k_fof_roots<<<nb, T, 0, s>>>(group, parent, n, least, status, cap);
     k_fof_least<<<nb, T, 0, s>>>(parent, n, least);
     k_fof_label<<<nb, T, 0, s>>>(sorted, parent, least, n, group);
     if (int rc = check_launch()) return rc;
